@@ -55,7 +55,18 @@ struct WindowDev {
   float bf[kMaxDim];        // the same two, rounded to float once (FP32 kernels)
   float kb_normf[kMaxDim];
   float binvf[kMaxDim];     // 1 / b in float (FP32 Gaussian)
+  // the window as polynomials (window_taps), per dimension [taps / 2][pairs];
+  // null for the B-spline
+  const float2* polyf[kMaxDim];
+  const double2* polyd[kMaxDim];
 };
+
+// Coefficient pairs of the window's polynomials: degree 11 in FP32, 21 in
+// FP64.  On a tap's unit interval the windows' Chebyshev coefficients fall
+// below 1e-9 and 1e-17 there for every cut-off and sigma up to 4 (the
+// narrowest windows need the highest degree).
+constexpr int kPolyF = 6;
+constexpr int kPolyD = 11;
 
 // psi(u) = phi(u / n) / phi(0) for the distance u (in cells).
 //   Gaussian:       exp(-u^2 / b)
@@ -143,6 +154,81 @@ __device__ __forceinline__ double window_psi<double>(const WindowDev& w, int t, 
   const double e = exp(-b * u2 / (z + m));
   const double s = -expm1(-2.0 * b * z) / z;
   return e * m * s * w.kb_norm[t];
+}
+
+// The W taps of a point at offset delta in [0, 1) of its cell, w[i] =
+// psi(delta + m - s - i), for the windows that are smooth inside their
+// support (all but the B-spline).  Tap i over its unit interval is a
+// polynomial in x = 2 delta - 1, and the window's symmetry makes tap W - 1 - i
+// the same one in -x: with E and O its even and odd parts in x^2, the two taps
+// are E + x O and E - x O.  Two FP32 taps cost 5 paired FMAs and 2 FMAs; the
+// formula (window_psi) costs 4 special-function instructions and about 16
+// others per tap, in FP64 about 110 FP64 operations against 11.  x is exact
+// to 2^-24 where u = delta + m - s would round at the size of m.  A window cut
+// at |u| = m is 0 there: its last tap at delta = 0.
+template <int W>
+__device__ __forceinline__ void window_taps(const WindowDev& win, int t, float delta, float* w) {
+  const float4* c = reinterpret_cast<const float4*>(win.polyf[t]);
+  const float x = fmaf(2.0f, delta, -1.0f);
+  const float s = x * x;
+#pragma unroll
+  for (int i = 0; i < W / 2; ++i) {
+    float2 p;
+#pragma unroll
+    for (int k = kPolyF / 2 - 1; k >= 0; --k) {
+      const float4 v = __ldg(c + i * (kPolyF / 2) + k);
+      if (k == kPolyF / 2 - 1) p = make_float2(v.z, v.w);
+      else p = cmad(p, s, make_float2(v.z, v.w));
+      p = cmad(p, s, make_float2(v.x, v.y));
+    }
+    w[i] = fmaf(x, p.y, p.x);
+    w[W - 1 - i] = fmaf(-x, p.y, p.x);
+  }
+  if (win.kind != 0 && delta == 0.0f) w[W - 1] = 0.0f;
+}
+template <int W>
+__device__ __forceinline__ void window_taps(const WindowDev& win, int t, double delta, double* w) {
+  const double2* c = win.polyd[t];
+  const double x = fma(2.0, delta, -1.0);
+  const double s = x * x;
+#pragma unroll
+  for (int i = 0; i < W / 2; ++i) {
+    double2 p = __ldg(c + i * kPolyD + kPolyD - 1);
+#pragma unroll
+    for (int k = kPolyD - 2; k >= 0; --k) p = cmad(p, s, __ldg(c + i * kPolyD + k));
+    w[i] = fma(x, p.y, p.x);
+    w[W - 1 - i] = fma(-x, p.y, p.x);
+  }
+  if (win.kind != 0 && delta == 0.0) w[W - 1] = 0.0;
+}
+
+// One of them, tap k (kernels whose lanes take different taps).
+__device__ __forceinline__ float window_tap(const WindowDev& win, int t, float delta, int k, int taps) {
+  const bool mirror = k >= taps / 2;
+  const float4* c = reinterpret_cast<const float4*>(win.polyf[t]) + (mirror ? taps - 1 - k : k) * (kPolyF / 2);
+  const float x = fmaf(2.0f, delta, -1.0f);
+  const float s = x * x;
+  float2 p;
+#pragma unroll
+  for (int q = kPolyF / 2 - 1; q >= 0; --q) {
+    const float4 v = __ldg(c + q);
+    if (q == kPolyF / 2 - 1) p = make_float2(v.z, v.w);
+    else p = cmad(p, s, make_float2(v.z, v.w));
+    p = cmad(p, s, make_float2(v.x, v.y));
+  }
+  if (win.kind != 0 && delta == 0.0f && k == taps - 1) return 0.0f;
+  return fmaf(mirror ? -x : x, p.y, p.x);
+}
+__device__ __forceinline__ double window_tap(const WindowDev& win, int t, double delta, int k, int taps) {
+  const bool mirror = k >= taps / 2;
+  const double2* c = win.polyd[t] + (mirror ? taps - 1 - k : k) * kPolyD;
+  const double x = fma(2.0, delta, -1.0);
+  const double s = x * x;
+  double2 p = __ldg(c + kPolyD - 1);
+#pragma unroll
+  for (int q = kPolyD - 2; q >= 0; --q) p = cmad(p, s, __ldg(c + q));
+  if (win.kind != 0 && delta == 0.0 && k == taps - 1) return 0.0;
+  return fma(mirror ? -x : x, p.y, p.x);
 }
 
 // Every window, the B-spline included (global kernels only).

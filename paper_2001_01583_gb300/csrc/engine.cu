@@ -197,6 +197,58 @@ double inv_c_at(int window, int m, int64_t n, double b, double k) {
 }
 
 
+namespace {
+
+// psi(u) of the kernels (common.cuh: window_psi).
+double window_psi_host(int window, int m, double b, double u) {
+  if (window == NFFT_GAUSSIAN) return std::exp(-u * u / b);
+  if (window == NFFT_SINC_POWER) {
+    const double x = M_PI * b * u;
+    return std::pow(x == 0.0 ? 1.0 : std::sin(x) / x, 2 * m);
+  }
+  const double z2 = (double)m * m - u * u;
+  const double z = z2 > 0.0 ? std::sqrt(z2) : 0.0;
+  const double s = z > 0.0 ? -std::expm1(-2.0 * b * z) / z : 2.0 * b;
+  return std::exp(-b * u * u / (z + m)) * m * s / (1.0 - std::exp(-2.0 * b * m));
+}
+
+// The polynomials of window_taps: for every tap of the first half the
+// Chebyshev interpolant of psi over its unit interval, x = 2 delta - 1, as
+// `pairs` coefficients of its even and odd parts in powers of x^2; appended
+// to `out` as the pairs lie in memory.
+template <typename Real>
+void append_window_polynomials(std::vector<double>& out, int window, int m, double b, int pairs) {
+  const int taps = taps_for(window, m), shift = window == NFFT_GAUSSIAN ? 0 : 1, n = 2 * pairs;
+  std::vector<double> cosines(4 * n);   // cos(pi q / 2n)
+  for (int q = 0; q < 4 * n; ++q) cosines[q] = std::cos(M_PI * q / (2.0 * n));
+  // Chebyshev polynomials in powers of x (integers below 2^53: exact)
+  std::vector<double> cheb((size_t)n * n, 0.0);
+  cheb[0] = 1.0;
+  cheb[n + 1] = 1.0;
+  for (int j = 2; j < n; ++j)
+    for (int k = 0; k < n; ++k)
+      cheb[(size_t)j * n + k] = (k > 0 ? 2.0 * cheb[(size_t)(j - 1) * n + k - 1] : 0.0) - cheb[(size_t)(j - 2) * n + k];
+  std::vector<Real> poly;
+  std::vector<double> y(n), mono(n);
+  for (int i = 0; i < taps / 2; ++i) {
+    for (int k = 0; k < n; ++k)
+      y[k] = window_psi_host(window, m, b, (cosines[2 * k + 1] + 1.0) / 2.0 + (double)(m - shift - i));
+    std::fill(mono.begin(), mono.end(), 0.0);
+    for (int j = 0; j < n; ++j) {
+      double c = 0.0;
+      for (int k = 0; k < n; ++k) c += y[k] * cosines[j * (2 * k + 1) % (4 * n)];
+      c *= (j == 0 ? 1.0 : 2.0) / n;
+      for (int k = j & 1; k <= j; k += 2) mono[k] += c * cheb[(size_t)j * n + k];
+    }
+    for (int k = 0; k < n; ++k) poly.push_back((Real)mono[k]);
+  }
+  const size_t at = out.size(), bytes = poly.size() * sizeof(Real);
+  out.resize(at + (bytes + 7) / 8);
+  std::memcpy(out.data() + at, poly.data(), bytes);
+}
+
+}  // namespace
+
 // ===========================================================================
 // parameters shared with nfft_plan_params
 
@@ -593,7 +645,12 @@ int Engine::build_layout() {
         const auto key = std::make_tuple(s.window, s.N[t], (int64_t)g.n[t], s.m, 0);
         auto f = table_cache.find(key);
         if (f == table_cache.end()) {
+          // the scaling table, then the window's polynomials (N is even: 16-byte aligned)
           std::vector<double> tab = scaling_table(s.window, s.m, s.N[t], g.n[t], b);
+          if (s.window != NFFT_B_SPLINE) {
+            if (precision == NFFT_FP64) append_window_polynomials<double>(tab, s.window, s.m, b, kPolyD);
+            else append_window_polynomials<float>(tab, s.window, s.m, b, kPolyF);
+          }
           double* dtab = nullptr;
           TRY(alloc_dev(dtab, sizeof(double) * tab.size(), device_bytes));
           CK(cudaMemcpy(dtab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
@@ -601,6 +658,10 @@ int Engine::build_layout() {
           f = table_cache.emplace(key, dtab).first;
         }
         it.inv_c[t] = f->second;
+        if (s.window != NFFT_B_SPLINE) {
+          w.polyf[t] = reinterpret_cast<const float2*>(f->second + s.N[t]);
+          w.polyd[t] = reinterpret_cast<const double2*>(f->second + s.N[t]);
+        }
       }
     }
     FClass& fc = fclasses[item_fclass[u]];

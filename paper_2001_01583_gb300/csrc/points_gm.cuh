@@ -53,8 +53,7 @@ __device__ __forceinline__ void gm_point(const SortedPoints<Real>& pts, const It
   __syncwarp();
   for (int i = lane; i < D * W; i += 32) {
     const int t = i / W, k = i - t * W;
-    const Real base = pts.delta[t][idx] + (Real)(it.win.m - it.win.shift);
-    wt[i] = window_psi<Real>(it.win, t, base - (Real)k);
+    wt[i] = window_tap(it.win, t, pts.delta[t][idx], k, W);
   }
   __syncwarp();
   int first[kMaxDim];

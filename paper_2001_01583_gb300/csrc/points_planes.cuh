@@ -220,47 +220,42 @@ __device__ __forceinline__ void plane_stage_batch(const PointKernelArgs<Real>& a
   rec.vx = 0;
   rec.vy = 0;
   Real* w = s.wt + (size_t)t * stride;
-  Real base[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) base[d] = a.pts.delta[d][idx] + (Real)(win.m - win.shift);
+  Real psi[W];
   if (NW == 0) {
     s.jt[t] = j;
     if constexpr (sizeof(Real) == 4 && W % 2 == 0) {
       // 8-byte stores (row stride 3W even, table 16-byte aligned)
       float2* w2 = reinterpret_cast<float2*>(w);
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
+      for (int d = 0; d < 3; ++d) {
+        window_taps<W>(win, d, a.pts.delta[d][idx], psi);
 #pragma unroll
-        for (int i = 0; i < W; i += 2)
-          w2[(d * W + i) / 2] = make_float2(window_psi<float>(win, d, base[d] - (float)i),
-                                            window_psi<float>(win, d, base[d] - (float)(i + 1)));
+        for (int i = 0; i < W; i += 2) w2[(d * W + i) / 2] = make_float2(psi[i], psi[i + 1]);
+      }
     } else {
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
+      for (int d = 0; d < 3; ++d) {
+        window_taps<W>(win, d, a.pts.delta[d][idx], psi);
 #pragma unroll
-        for (int i = 0; i < W; ++i) w[d * W + i] = window_psi<Real>(win, d, base[d] - (Real)i);
+        for (int i = 0; i < W; ++i) w[d * W + i] = psi[i];
+      }
     }
   } else {
     using R = SpreadRow<W, (NW > 0 ? NW : 1)>;
     constexpr int NWs = NW > 0 ? NW : 1;
+    window_taps<W>(win, 0, a.pts.delta[0][idx], psi);
 #pragma unroll
-    for (int u = 0; u < R::TAPS; ++u)
+    for (int i = 0; i < W; ++i) {
+      // tap i is the (i / NW)-th of warp (l0 + i) mod NW
+      const int slot = R::ROT ? i / NWs * NWs + ((l0 + i) & (NWs - 1)) : i;
+      w[R::WZ + slot] = psi[i];
+    }
+    window_taps<W>(win, 1, a.pts.delta[1][idx], psi);
 #pragma unroll
-      for (int ww = 0; ww < NWs; ++ww) {
-        const int slot = u * NWs + ww;
-        const int i = R::ROT ? ((ww - l0) & (NWs - 1)) + u * NWs : slot;
-        if (slot < W) w[R::WZ + slot] = window_psi<Real>(win, 0, base[0] - (Real)i);
-      }
+    for (int i = 0; i < W; ++i) w[R::WY + (R::PERM ? i % S::Q * S::PASSES + i / S::Q : i)] = psi[i];
+    window_taps<W>(win, 2, a.pts.delta[2][idx], psi);
 #pragma unroll
-    for (int q = 0; q < S::Q; ++q)
-#pragma unroll
-      for (int k = 0; k < S::PASSES; ++k) {
-        const int slot = R::PERM ? q * S::PASSES + k : k * S::Q + q;
-        const int i = k * S::Q + q;
-        if (i < W) w[R::WY + slot] = window_psi<Real>(win, 1, base[1] - (Real)i);
-      }
-#pragma unroll
-    for (int i = 0; i < W; ++i) w[R::WX + i] = window_psi<Real>(win, 2, base[2] - (Real)i);
+    for (int i = 0; i < W; ++i) w[R::WX + i] = psi[i];
     if (NW < 0) {
       s.jt[t] = j;
     } else {
@@ -457,15 +452,10 @@ __device__ __forceinline__ void plane_stage_flat(const PointKernelArgs<float>& a
   const float2 v0 = f_in[(int64_t)r0 * M + j];
   rec.vx = v0.x;
   rec.vy = v0.y;
-  float base[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) base[d] = a.pts.delta[d][idx] + (float)(win.m - win.shift);
-  float wz[W], wy[W];
-#pragma unroll
-  for (int i = 0; i < W; ++i) {
-    wz[i] = window_psi<float>(win, 0, base[0] - (float)i);
-    wy[i] = window_psi<float>(win, 1, base[1] - (float)i);
-  }
+  float wz[W], wy[W], wx[W];
+  window_taps<W>(win, 0, a.pts.delta[0][idx], wz);
+  window_taps<W>(win, 1, a.pts.delta[1][idx], wy);
+  window_taps<W>(win, 2, a.pts.delta[2][idx], wx);
   // products first (16-byte stores: the row stride is an odd number of
   // 16-byte units and the table 16-byte aligned), then wx
   using F = FlatShape<W, NW>;
@@ -493,8 +483,7 @@ __device__ __forceinline__ void plane_stage_flat(const PointKernelArgs<float>& a
   }
 #pragma unroll
   for (int i = 0; i < W; i += 2)
-    *reinterpret_cast<float2*>(w + F::WX + i) = make_float2(window_psi<float>(win, 2, base[2] - (float)i),
-                                                            window_psi<float>(win, 2, base[2] - (float)(i + 1)));
+    *reinterpret_cast<float2*>(w + F::WX + i) = make_float2(wx[i], wx[i + 1]);
   s.rec[t] = rec;
 }
 
@@ -815,9 +804,9 @@ __device__ __forceinline__ void interp_points_fast(const PlaneSmem<W, Real>& s, 
   }
 }
 
-// FP32 narrow windows: three blocks of 256 threads per SM (at most 85 registers)
+// narrow windows: three blocks of 256 threads per SM in FP32 (at most 85 registers), two in FP64
 template <int W, typename Real>
-__global__ void __launch_bounds__(256, (W <= 8 && sizeof(Real) == 4) ? 3 : 1) k_interp_groups(PointKernelArgs<Real> a, WppLayout lay) {
+__global__ void __launch_bounds__(256, W > 8 ? 1 : (sizeof(Real) == 4 ? 3 : 2)) k_interp_groups(PointKernelArgs<Real> a, WppLayout lay) {
   using C = typename Cplx<Real>::type;
   using S = PlaneShape<W>;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -57,9 +57,7 @@ __device__ __forceinline__ int64_t tile_to_grid(int e, const GridGeom& g, const 
 
 template <int W, typename Real>
 __device__ __forceinline__ void taps_of(const WindowDev& win, int t, Real delta, Real* w) {
-  const Real base = delta + (Real)(win.m - win.shift);
-#pragma unroll
-  for (int i = 0; i < W; ++i) w[i] = window_psi<Real>(win, t, base - (Real)i);
+  window_taps<W>(win, t, delta, w);
 }
 
 template <int D, int W, typename Real>

@@ -59,9 +59,10 @@ __device__ __forceinline__ WppBatch<D, W, Real> wpp_load_batch(const PointKernel
     Real* w = wtab + lane * (D * W);
 #pragma unroll
     for (int t = 0; t < D; ++t) {
-      const Real base = a.pts.delta[t][idx] + (Real)(win.m - win.shift);
+      Real psi[W];
+      window_taps<W>(win, t, a.pts.delta[t][idx], psi);
 #pragma unroll
-      for (int i = 0; i < W; ++i) w[t * W + i] = window_psi<Real>(win, t, base - (Real)i);
+      for (int i = 0; i < W; ++i) w[t * W + i] = psi[i];
     }
   }
   __syncwarp();
