@@ -244,6 +244,7 @@ struct SubProblem {
   int start;   // first sorted position
   int count;
   int item;
+  int dense;   // pencils: points share cells (kDenseRun of them per cell or more)
 };
 
 struct GridGeom {
@@ -254,6 +255,7 @@ struct GridGeom {
   int tile[kMaxDim];         // bin + W - 1 (unused dims = 1)
   int64_t grid_cells;        // prod n
   int tile_cells;            // prod tile
+  int fine;                  // sort keys per bin: 1, or bin[0] (a bin's points in the order of their plane)
 };
 
 // One transform of a batch (a single plan is a batch of one), as the
@@ -268,6 +270,7 @@ struct ItemDev {
   int64_t M;
   int nrhs;
   int bin_offset;              // first global bin id of the item
+  int key_offset;              // first sort key of the item (geom.fine keys per bin)
   int64_t point_offset;        // first point of the item in the unsorted concatenation
   const double* x;             // M x d points (read by nfft_set_points only)
   void* grid;                  // nrhs grids of geom.grid_cells

@@ -12,6 +12,7 @@ namespace gbnfft {
 namespace {
 
 constexpr size_t kSmemBudget = 200 * 1024;   // per block (the opt-in limit is 227 KB)
+constexpr int kPencilBlocksPerSm = 16;       // pencil subproblems per SM a point set is cut into at least
 constexpr size_t kSmemTarget = 100 * 1024;   // thread-per-point tiles: aim at two blocks per SM
 
 #define CK(call)                                                             \
@@ -404,6 +405,8 @@ int Engine::release_layout() {
   free_dev(d_bin_offsets);
   free_dev(d_crop_blocks);
   free_dev(d_pad_blocks);
+  free_dev(key_count);
+  free_dev(key_start);
   free_dev(bin_count);
   free_dev(bin_start);
   free_dev(sub_count);
@@ -411,7 +414,7 @@ int Engine::release_layout() {
   free_dev(scan_partials);
   free_dev(num_subs);
   free_dev(subs);
-  free_dev(bin_rank);
+  free_dev(key_rank);
   free_dev(perm);
   free_dev(local);
   for (int t = 0; t < 3; ++t) free_dev(delta[t]);
@@ -433,9 +436,10 @@ int Engine::build_layout() {
 
   struct Choice {
     int bin[3], tile[3], pitch, method, taps, sparse, sparse_interp;
-    bool owner, tensor, tensor_interp;
+    bool owner, tensor, tensor_interp, pencil;
   };
   std::vector<Choice> ch(nitems);
+  bool any_pencil = false;
   for (int i = 0; i < nitems; ++i) {
     const ItemSpec& s = specs[i];
     Choice& c = ch[i];
@@ -553,6 +557,28 @@ int Engine::build_layout() {
     // 3-D sparse bins spread by their cells' owners (no atomics): needs one
     // periodic image per footprint (n_t >= bin_t + W - 1) and the warps'
     // tiles in shared memory
+    // pencils (points_pencil.cuh): 3-D items in FP32 with nothing chosen by
+    // the caller that belongs to the other kernels (method, bins, split, owner
+    // or tensor-core form), and at least a point per plane of a pencil on
+    // average.  Below that the window moves on with every point and is written
+    // out for it alone, as the grid-warp kernels do without sorting by plane:
+    // N = 64^3, 8 taps, one set: 20,000 points (0.8 per plane) take 174 us in
+    // pencils and 166 us on the other kernels, 96,000 points (3.7) 19 us
+    // against 36 to spread and 72 against 103 to interpolate one right-hand side.
+    const PencilLaunch pl = pencil_launch_f32(c.taps, true);
+    c.pencil = s.d == 3 && method_opt == NFFT_METHOD_AUTO && method == NFFT_METHOD_WARP &&
+               precision == NFFT_FP32_MIXED && !explicit_bins && sparse_opt == 0 && sparse_interp_opt == 0 &&
+               !owner_enabled && !c.tensor && !c.tensor_interp && pl.fn &&
+               (double)s.M * pl.edge * pl.edge >= (double)n[0] * (double)n[1] * (double)n[2];
+    if (c.pencil) {
+      const int want[3] = {(1 << local_bits(3)) - 1, pl.edge, pl.edge};
+      for (int t = 0; t < 3; ++t) {
+        c.bin[t] = (int)std::min<int64_t>(want[t], n[t]);
+        c.tile[t] = c.bin[t] + c.taps - 1;
+      }
+      c.sparse = c.sparse_interp = 0;
+      any_pencil = true;
+    }
     c.owner = false;
     if (s.d == 3 && c.sparse > 0 && owner_enabled) {
       const bool built = (precision == NFFT_FP64 ? owner_kernel_f64(c.taps) : owner_kernel_f32(c.taps)) != nullptr;
@@ -567,6 +593,12 @@ int Engine::build_layout() {
       c.owner = fits && osmem <= smem_optin;
     }
   }
+  if (any_pencil && max_sub_opt == 0) {
+    int64_t total = 0;
+    for (const auto& s : specs) total += s.M;
+    const int64_t want = total / ((int64_t)num_sms * kPencilBlocksPerSm);
+    max_sub = (int)std::min<int64_t>(1024, std::max<int64_t>(32, (want + 31) / 32 * 32));
+  }
   // group items into kernel classes (stable by first appearance)
   // (items with different right-hand-side counts get their own launch: the
   // right-hand sides per pass size the shared memory of the whole launch)
@@ -574,7 +606,7 @@ int Engine::build_layout() {
     return specs[a].d == specs[b].d && ch[a].taps == ch[b].taps && specs[a].window == specs[b].window &&
            (single || specs[a].nrhs == specs[b].nrhs) &&
            ch[a].method == ch[b].method && ch[a].sparse == ch[b].sparse &&
-           ch[a].sparse_interp == ch[b].sparse_interp && ch[a].owner == ch[b].owner && ch[a].bin[0] == ch[b].bin[0] &&
+           ch[a].sparse_interp == ch[b].sparse_interp && ch[a].owner == ch[b].owner && ch[a].pencil == ch[b].pencil && ch[a].bin[0] == ch[b].bin[0] &&
            ch[a].bin[1] == ch[b].bin[1] &&
            ch[a].bin[2] == ch[b].bin[2];
   };
@@ -600,6 +632,7 @@ int Engine::build_layout() {
   kclasses.clear();
   std::vector<int64_t> pts_off(nitems + 1, 0);
   std::vector<int> bin_off(nitems + 1, 0);
+  int64_t keys = 0;
   max_subs_total = 0;
   for (int k = 0; k < nitems; ++k) {
     const int u = order[k];
@@ -623,6 +656,7 @@ int Engine::build_layout() {
       nb_total *= g.nbins[t];
       it.N[t] = t < s.d ? (int)s.N[t] : 1;
     }
+    g.fine = c.pencil ? c.bin[0] : 1;
     it.NN = 1;
     for (int t = 0; t < s.d; ++t) it.NN *= s.N[t];
     it.M = s.M;
@@ -668,10 +702,12 @@ int Engine::build_layout() {
     it.grid = static_cast<char*>(fc.buf) + item_grid_offset[u] * (int64_t)csize;
     it.point_offset = pts_off[k];
     it.bin_offset = bin_off[k];
+    it.key_offset = (int)keys;
+    keys += (int64_t)nb_total * g.fine;
     pts_off[k + 1] = pts_off[k] + s.M;
     bin_off[k + 1] = bin_off[k] + nb_total;
     max_subs_total += nb_total + s.M / max_sub + 1;
-    if ((int64_t)bin_off[k + 1] > ((int64_t)1 << 30)) return NFFT_ERR_UNSUPPORTED;
+    if ((int64_t)bin_off[k + 1] > ((int64_t)1 << 30) || keys > ((int64_t)1 << 30)) return NFFT_ERR_UNSUPPORTED;
     // kernel class bookkeeping
     if (kclasses.empty() || cls[u] != cls[order[kclasses.back().item_begin]]) {
       KClass kc{};
@@ -687,6 +723,7 @@ int Engine::build_layout() {
       kc.sparse_points = c.sparse;
       kc.sparse_points_interp = c.sparse_interp;
       kc.owner = c.owner;
+      kc.pencil = c.pencil;
       kc.tensor = c.tensor;
       kc.tensor_interp = c.tensor_interp;
       kc.item_begin = k;
@@ -710,20 +747,24 @@ int Engine::build_layout() {
     for (int k = kc.item_begin; k < kc.item_end; ++k)
       if (!kc.owner) fclasses[item_fclass[order[k]]].owner_written = false;
   total_bins = bin_off[nitems];
+  total_keys = (int)keys;
   // device buffers
   int64_t before = device_bytes;
   const size_t P = (size_t)std::max<int64_t>(total_points, 1);
   const size_t B = (size_t)std::max(total_bins, 1);
   TRY(alloc_dev(d_point_offsets, sizeof(int64_t) * (nitems + 1), device_bytes));
   TRY(alloc_dev(d_bin_offsets, sizeof(int) * (nitems + 1), device_bytes));
+  const size_t K = (size_t)std::max(total_keys, 1);
+  TRY(alloc_dev(key_count, sizeof(int) * K, device_bytes));
+  TRY(alloc_dev(key_start, sizeof(int) * (K + 1), device_bytes));
   TRY(alloc_dev(bin_count, sizeof(int) * B, device_bytes));
   TRY(alloc_dev(bin_start, sizeof(int) * B, device_bytes));
   TRY(alloc_dev(sub_count, sizeof(int) * B, device_bytes));
   TRY(alloc_dev(sub_start, sizeof(int) * B, device_bytes));
-  TRY(alloc_dev(scan_partials, sizeof(int) * (size_t)scan_partials_needed((int)B), device_bytes));
+  TRY(alloc_dev(scan_partials, sizeof(int) * (size_t)scan_partials_needed((int)std::max(B, K)), device_bytes));
   TRY(alloc_dev(num_subs, sizeof(int), device_bytes));
   TRY(alloc_dev(subs, sizeof(SubProblem) * (size_t)max_subs_total, device_bytes));
-  TRY(alloc_dev(bin_rank, sizeof(int2) * P, device_bytes));
+  TRY(alloc_dev(key_rank, sizeof(int2) * P, device_bytes));
   TRY(alloc_dev(perm, sizeof(int) * P, device_bytes));
   TRY(alloc_dev(local, sizeof(uint32_t) * P, device_bytes));
   const int dmax = [&] {
@@ -978,6 +1019,8 @@ int Engine::run_points(const KClass& kc, bool spread, const void* in, void* out,
   a.sub_min_count = 0;
   a.sub_max_count = INT_MAX;
   a.err = err_flag;
+  if constexpr (sizeof(Real) == 4)
+    if (kc.pencil) return run_pencil(kc, a, spread, max_nrhs);
   if (kc.method == NFFT_METHOD_GRID_WARP) return run_gm<Real>(kc, a, spread);
   if (kc.method == NFFT_METHOD_GLOBAL) return run_global<Real>(kc, a, spread);
   // tiled kernels take the bins of at least `split` points, the owner
@@ -1096,6 +1139,20 @@ int Engine::run_planes(const KClass& kc, PointKernelArgs<Real>& a, bool spread, 
   CK(cudaLaunchKernel(best_fn, dim3((unsigned)blocks), dim3(32 * best_nw), args, best_smem, stream));
   ++kernel_launches;
   (spread ? last_spread_threads : last_interp_threads) = 32 * best_nw;
+  return NFFT_OK;
+}
+
+// 3-D pencils (points_pencil.cuh): a block per subproblem and right-hand
+// side; the grid is the bound on the subproblems, blocks past the last return.
+int Engine::run_pencil(const KClass& kc, PointKernelArgs<float>& a, bool spread, int max_nrhs) {
+  const PencilLaunch l = pencil_launch_f32(kc.taps, spread);
+  a.rhs_per_pass = 1;
+  const dim3 blocks((unsigned)std::max<int64_t>(kc.max_subs, 1), (unsigned)max_nrhs);
+  void* args[] = {&a};
+  CK(cudaFuncSetAttribute(l.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem));
+  CK(cudaLaunchKernel(l.fn, blocks, dim3(l.threads), args, l.smem, stream));
+  ++kernel_launches;
+  (spread ? last_spread_threads : last_interp_threads) = l.threads;
   return NFFT_OK;
 }
 
@@ -1243,16 +1300,24 @@ int Engine::set_points_impl(const double* x_override) {
   s.single_d = items.size() == 1 ? items[0].geom.d : 0;
   EventPair ev{};
   TRY(stage_begin(NFFT_STAGE_SORT, &ev));
-  CK(cudaMemsetAsync(bin_count, 0, sizeof(int) * (size_t)std::max(total_bins, 1), stream));
-  CK(launch_bin_count<Real>(s, bin_count, bin_rank, stream));
-  // bin count, scatter, subproblem count and fill, two scans
-  kernel_launches += (s.total_points > 0 ? 4 : 2) + 2 * scan_launches(total_bins);
-  CK(launch_scan(bin_count, bin_start, total_bins, nullptr, scan_partials, stream));
+  CK(cudaMemsetAsync(key_count, 0, sizeof(int) * (size_t)std::max(total_keys, 1), stream));
+  CK(launch_key_count<Real>(s, key_count, key_rank, stream));
+  // key count, scatter, subproblem count and fill, two scans
+  kernel_launches += (s.total_points > 0 ? 4 : 2) + scan_launches(total_keys) + scan_launches(total_bins);
+  CK(launch_scan(key_count, key_start, total_keys, key_start + total_keys, scan_partials, stream));
   Real* d[3] = {static_cast<Real*>(delta[0]), static_cast<Real*>(delta[1]), static_cast<Real*>(delta[2])};
-  CK(launch_scatter<Real>(s, bin_start, bin_rank, perm, local, d, stream));
-  CK(launch_subproblem_count(bin_count, total_bins, max_sub, sub_count, stream));
+  CK(launch_scatter<Real>(s, key_start, key_rank, perm, local, d, stream));
+  CK(launch_subproblem_count(s, key_start, max_sub, bin_count, bin_start, sub_count, stream));
   CK(launch_scan(sub_count, sub_start, total_bins, num_subs, scan_partials, stream));
   CK(launch_subproblem_fill(s, bin_count, bin_start, sub_start, max_sub, subs, stream));
+  if constexpr (sizeof(Real) == 4) {
+    bool pencils = false;
+    for (const auto& kc : kclasses) pencils = pencils || kc.pencil;
+    if (pencils && s.total_points > 0) {
+      CK(launch_refine(s, max_subs_total, subs, num_subs, perm, local, d, stream));
+      ++kernel_launches;
+    }
+  }
   TRY(stage_end(&ev));
   return NFFT_OK;
 }
@@ -1820,6 +1885,8 @@ int Engine::autotune(int reps, double* best_ms) {
     const int bins[][3] = {{8, 8, 16}, {8, 8, 8}, {4, 8, 16}, {8, 16, 16}, {8, 8, 32}, {4, 4, 32}};
     for (const auto& b : bins)
       for (int P : Ps) cands.push_back(Cand{{b[0], b[1], b[2]}, P});
+    // the automatic layout (pencils in FP32)
+    for (int P : Ps) cands.push_back(Cand{{0, 0, 0}, P});
   } else if (dmax == 2) {
     const int bins[][2] = {{32, 32}, {16, 32}, {32, 64}, {64, 64}, {16, 16}};
     for (const auto& b : bins)

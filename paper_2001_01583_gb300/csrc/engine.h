@@ -41,6 +41,7 @@ struct KClass {
   int64_t max_subs;           // bound on the class's subproblems
   int sparse_points;          // spreading subproblems below this many points: grid-warp kernel (0: none)
   int sparse_points_interp;   // the same for interpolation
+  bool pencil;                // 3-D FP32 pencils (points_pencil.cuh)
   bool owner;                 // spreading of sparse bins by the owner kernel (3-D)
   bool tensor;                // dense bins spread on the tensor cores (3-D, FP32)
   bool tensor_interp;         // dense bins interpolated on the tensor cores (3-D, FP32)
@@ -125,6 +126,7 @@ class Engine {
   template <typename Real> int run_gm(const KClass& kc, PointKernelArgs<Real>& a, bool spread);
   template <typename Real> int run_owner(const KClass& kc, PointKernelArgs<Real>& a);
   template <typename Real> int run_global(const KClass& kc, PointKernelArgs<Real>& a, bool spread);
+  int run_pencil(const KClass& kc, PointKernelArgs<float>& a, bool spread, int max_nrhs);
   int run_tc(const KClass& kc, PointKernelArgs<float>& a, bool spread);
   template <typename Real> int adjoint_table(bool in_graph);
   template <typename Real> int forward_table(bool in_graph);
@@ -188,12 +190,15 @@ class Engine {
   // sort buffers
   int64_t total_points = 0;
   int total_bins = 0;
+  int total_keys = 0;             // sort keys (GridGeom::fine per bin)
   int64_t max_subs_total = 0;
   int64_t* d_point_offsets = nullptr;
   int* d_bin_offsets = nullptr;
   int* d_crop_blocks = nullptr;        // scaling launches: per-item block prefix sums, then each block's item
   int* d_pad_blocks = nullptr;
   int64_t crop_blocks = 0, pad_blocks = 0;
+  int* key_count = nullptr;       // points per sort key, and their exclusive scan
+  int* key_start = nullptr;
   int* bin_count = nullptr;
   int* bin_start = nullptr;
   int* sub_count = nullptr;
@@ -201,7 +206,7 @@ class Engine {
   int* sub_start = nullptr;
   int* num_subs = nullptr;
   SubProblem* subs = nullptr;
-  int2* bin_rank = nullptr;
+  int2* key_rank = nullptr;
   int* perm = nullptr;
   uint32_t* local = nullptr;
   void* delta[3] = {nullptr, nullptr, nullptr};

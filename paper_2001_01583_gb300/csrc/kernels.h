@@ -25,9 +25,11 @@ struct SortArgs {
   int* err;                       // bit 0: non-finite coordinate
   int single_d;                   // one item: its dimension (the kernels' one-item form); 0 otherwise
 };
-// Cell and global bin of every point, and its rank inside its bin.
+// Sort keys: item i's bins in order, GridGeom::fine keys each (fine > 1: one
+// per plane of the bin along dimension 0); item i's keys start at key_offset.
+// Key of every point, its rank among the points of its key, and the keys' counts.
 template <typename Real>
-cudaError_t launch_bin_count(const SortArgs& s, int* bin_count, int2* bin_rank, cudaStream_t st);
+cudaError_t launch_key_count(const SortArgs& s, int* key_count, int2* key_rank, cudaStream_t st);
 // Exclusive prefix sum of n ints; *total = sum (may be null).  partials:
 // scan_partials_needed(n) ints of device scratch.  scan_launches(n) kernels.
 int scan_partials_needed(int n);
@@ -35,12 +37,20 @@ int scan_launches(int n);
 cudaError_t launch_scan(const int* in, int* out, int n, int* total, int* partials, cudaStream_t st);
 // Write every point to its sorted slot: perm (index within its item), packed in-bin offsets, deltas.
 template <typename Real>
-cudaError_t launch_scatter(const SortArgs& s, const int* bin_start, const int2* bin_rank, int* perm, uint32_t* local,
+cudaError_t launch_scatter(const SortArgs& s, const int* key_start, const int2* key_rank, int* perm, uint32_t* local,
                            Real* const* delta, cudaStream_t st);
-// Subproblems per global bin (ceil(count / P)), then their records.
-cudaError_t launch_subproblem_count(const int* bin_count, int nbins, int P, int* sub_count, cudaStream_t st);
+// Points, first sorted position and subproblems (ceil(count / P)) of every
+// global bin from its keys (key_start: their exclusive scan, one past the end
+// too), then the subproblems' records.
+cudaError_t launch_subproblem_count(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
+                                    int* sub_count, cudaStream_t st);
 cudaError_t launch_subproblem_fill(const SortArgs& s, const int* bin_count, const int* bin_start, const int* sub_start,
                                    int P, SubProblem* subs, cudaStream_t st);
+
+// Pencil items (GridGeom::fine > 1): the points of every subproblem ordered by
+// cell and their records written (the scatter writes their indices only).
+cudaError_t launch_refine(const SortArgs& s, int64_t max_subs, SubProblem* subs, const int* num_subs, int* perm,
+                          uint32_t* local, float* const* delta, cudaStream_t st);
 
 // ---- spreading / interpolation ---------------------------------------------
 template <typename Real>
@@ -128,6 +138,18 @@ const void* planes_kernel_f32(int taps, int warps, bool spread);
 const void* planes_kernel_f64(int taps, int warps, bool spread);
 size_t planes_table_bytes_f32(int taps, int bp, int np, int nw, const int* tile, bool spread);
 size_t planes_table_bytes_f64(int taps, int bp, int np, int nw, const int* tile, bool spread);
+
+// 3-D pencil kernels (points_pencil.cuh): FP32, even windows of up to 16 taps;
+// a block of `threads` per subproblem (grid.x) and right-hand side (grid.y),
+// pencils of edge x edge cells in dimensions 1 and 2, points sorted by plane.
+struct PencilLaunch {
+  const void* fn;   // null: not built
+  int threads;
+  size_t smem;
+  int edge;
+};
+PencilLaunch pencil_launch_f32(int taps, bool spread);
+constexpr int kDenseRun = 4;   // points per occupied cell from which a pencil's subproblem is dense
 
 // 3-D spreading on the tensor cores (points_tc.cuh): FP32, taps 4, 6 or 8,
 // tiles of at most 128 (z, y) rows and 2 T2 <= kTcMaxColsHost real columns;

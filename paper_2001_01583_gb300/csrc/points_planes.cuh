@@ -698,12 +698,11 @@ __global__ void __launch_bounds__(32 * NW) k_spread_planes(PointKernelArgs<Real>
 }
 
 // The 4 points' 8 real values of a warp pass (v[2g], v[2g + 1]: this lane's
-// share of point p0 + g), reduced over the warp at once by a transposed
-// butterfly (10 shuffles): after the exchanges over lane bits 4, 3 and 2 each
-// lane keeps one value, and bits 1 and 0 finish its sum; lane 8g then
-// writes point p0 + g to its place in the caller's order.
-__device__ __forceinline__ void butterfly4_store(const float* v, int lane, int p0, int nb, uint32_t jt_a,
-                                                 float2* out) {
+// share of point g), reduced over the warp at once by a transposed
+// butterfly (9 shuffles): after the exchanges over lane bits 4, 3 and 2 each
+// lane keeps one value, and bits 1 and 0 finish its sum.  Lane l returns the
+// sum of value l >> 2.
+__device__ __forceinline__ float butterfly8(const float* v, int lane) {
   const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
   float a4[4], a2[2];
 #pragma unroll
@@ -726,12 +725,19 @@ __device__ __forceinline__ void butterfly4_store(const float* v, int lane, int p
   }
   a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
   a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
-  // lane l now holds value l >> 2: point l >> 3, real part when bit 2 is 0
-  const float im = __shfl_down_sync(0xffffffffu, a1, 4);
+  return a1;
+}
+
+// butterfly8 of points p0 .. p0 + 3: lane 8g writes point p0 + g to its place in the caller's order.
+__device__ __forceinline__ void butterfly4_store(const float* v, int lane, int p0, int nb, uint32_t jt_a,
+                                                 float2* out) {
+  const float re = butterfly8(v, lane);
+  // value l >> 2 is point l >> 3, its real part when bit 2 is 0
+  const float im = __shfl_down_sync(0xffffffffu, re, 4);
   const int g = lane >> 3;
   if ((lane & 7) == 0 && p0 + g < nb) {
     const int j = lds_i1(jt_a + 4u * (uint32_t)(p0 + g));
-    out[j] = make_float2(a1, im);
+    out[j] = make_float2(re, im);
   }
 }
 

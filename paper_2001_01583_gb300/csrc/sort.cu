@@ -105,16 +105,16 @@ constexpr int kSortThreads = 256;
 constexpr int kSortPer = 4;
 
 template <typename Real>
-__global__ void __launch_bounds__(kSortThreads) k_bin_count(SortArgs s, int* __restrict__ bin_count,
-                                                            int2* __restrict__ bin_rank) {
+__global__ void __launch_bounds__(kSortThreads) k_key_count(SortArgs s, int* __restrict__ key_count,
+                                                            int2* __restrict__ key_rank) {
   const int64_t base = (int64_t)blockIdx.x * (kSortThreads * kSortPer) + threadIdx.x;
   const int lane = threadIdx.x & 31;
-  int bin[kSortPer];
+  int key[kSortPer];
   bool any_bad = false;
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int64_t gidx = base + (int64_t)k * kSortThreads;
-    bin[k] = -1;
+    key[k] = -1;
     if (gidx < s.total_points) {
       const int item = find_item<int64_t>(s.point_offsets, s.n_items, gidx);
       const ItemDev& it = s.items[item];
@@ -122,15 +122,17 @@ __global__ void __launch_bounds__(kSortThreads) k_bin_count(SortArgs s, int* __r
       const double* x = s.x_override ? s.x_override : it.x;
       const GridGeom& g = it.geom;
       bool bad = false;
-      int local = 0;
+      int local = 0, plane = 0;
       for (int t = 0; t < g.d; ++t) {
         int c;
         Real dl;
         reduce_coord<Real>(load_coord(x, j, g.d, t, bad), g.n[t], c, dl);
-        local = local * g.nbins[t] + c / g.bin[t];
+        const int b = c / g.bin[t];
+        if (t == 0) plane = c - b * g.bin[0];
+        local = local * g.nbins[t] + b;
       }
       any_bad |= bad;
-      bin[k] = it.bin_offset + local;
+      key[k] = it.key_offset + local * g.fine + (g.fine > 1 ? plane : 0);
     }
   }
   if (any_bad) atomicOr(s.err, 1);
@@ -140,21 +142,21 @@ __global__ void __launch_bounds__(kSortThreads) k_bin_count(SortArgs s, int* __r
   int got[kSortPer];
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
-    peers[k] = __match_any_sync(0xffffffffu, bin[k]);
+    peers[k] = __match_any_sync(0xffffffffu, key[k]);
     got[k] = 0;
-    if (bin[k] >= 0 && lane == __ffs(peers[k]) - 1) got[k] = atomicAdd(&bin_count[bin[k]], __popc(peers[k]));
+    if (key[k] >= 0 && lane == __ffs(peers[k]) - 1) got[k] = atomicAdd(&key_count[key[k]], __popc(peers[k]));
   }
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int first = __shfl_sync(peers[k], got[k], __ffs(peers[k]) - 1);
     const int64_t gidx = base + (int64_t)k * kSortThreads;
-    if (bin[k] >= 0) bin_rank[gidx] = make_int2(bin[k], first + __popc(peers[k] & ((1u << lane) - 1u)));
+    if (key[k] >= 0) key_rank[gidx] = make_int2(key[k], first + __popc(peers[k] & ((1u << lane) - 1u)));
   }
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(kSortThreads) k_scatter(SortArgs s, const int* __restrict__ bin_start,
-                                                          const int2* __restrict__ bin_rank, int* __restrict__ perm,
+__global__ void __launch_bounds__(kSortThreads) k_scatter(SortArgs s, const int* __restrict__ key_start,
+                                                          const int2* __restrict__ key_rank, int* __restrict__ perm,
                                                           uint32_t* __restrict__ local, Real* d0, Real* d1, Real* d2) {
   const int64_t base = (int64_t)blockIdx.x * (kSortThreads * kSortPer) + threadIdx.x;
   Real* dst[3] = {d0, d1, d2};
@@ -163,10 +165,10 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(SortArgs s, const int*
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int64_t gidx = base + (int64_t)k * kSortThreads;
-    br[k] = gidx < s.total_points ? bin_rank[gidx] : make_int2(-1, 0);
+    br[k] = gidx < s.total_points ? key_rank[gidx] : make_int2(-1, 0);
   }
 #pragma unroll
-  for (int k = 0; k < kSortPer; ++k) pos[k] = br[k].x >= 0 ? bin_start[br[k].x] + br[k].y : -1;
+  for (int k = 0; k < kSortPer; ++k) pos[k] = br[k].x >= 0 ? key_start[br[k].x] + br[k].y : -1;
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int64_t gidx = base + (int64_t)k * kSortThreads;
@@ -176,6 +178,8 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(SortArgs s, const int*
     const int64_t j = gidx - it.point_offset;
     const double* x = s.x_override ? s.x_override : it.x;
     const GridGeom& g = it.geom;
+    perm[pos[k]] = (int)j;
+    if (g.fine > 1) continue;   // k_refine writes the rest
     bool bad = false;
     uint32_t packed = 0;
     const int bits = local_bits(g.d);
@@ -187,7 +191,6 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(SortArgs s, const int*
       packed |= (g.d == 1) ? lc : (lc << (bits * t));
       dst[t][pos[k]] = dl;
     }
-    perm[pos[k]] = (int)j;
     local[pos[k]] = packed;
   }
 }
@@ -200,13 +203,14 @@ template <int D>
 struct OneItem {
   const double* x;
   int64_t poff;
-  int boff;
+  int koff, fine;
   int n[D], bw[D], nb[D];
   __device__ __forceinline__ explicit OneItem(const SortArgs& s) {
     const ItemDev& it = s.items[0];
     x = s.x_override ? s.x_override : it.x;
     poff = it.point_offset;
-    boff = it.bin_offset;
+    koff = it.key_offset;
+    fine = it.geom.fine;
 #pragma unroll
     for (int t = 0; t < D; ++t) {
       n[t] = it.geom.n[t];
@@ -217,8 +221,8 @@ struct OneItem {
 };
 
 template <typename Real, int D>
-__global__ void __launch_bounds__(kSortThreads) k_bin_count_one(SortArgs s, int* __restrict__ bin_count,
-                                                                int2* __restrict__ bin_rank) {
+__global__ void __launch_bounds__(kSortThreads) k_key_count_one(SortArgs s, int* __restrict__ key_count,
+                                                                int2* __restrict__ key_rank) {
   const int64_t base = (int64_t)blockIdx.x * (kSortThreads * kSortPer) + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const OneItem<D> one(s);
@@ -229,12 +233,12 @@ __global__ void __launch_bounds__(kSortThreads) k_bin_count_one(SortArgs s, int*
 #pragma unroll
     for (int t = 0; t < D; ++t) v[k][t] = gidx < s.total_points ? one.x[(gidx - one.poff) * D + t] : 0.0;
   }
-  int bin[kSortPer];
+  int key[kSortPer];
   bool any_bad = false;
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int64_t gidx = base + (int64_t)k * kSortThreads;
-    int local = 0;
+    int local = 0, plane = 0;
 #pragma unroll
     for (int t = 0; t < D; ++t) {
       double c0 = v[k][t];
@@ -245,52 +249,57 @@ __global__ void __launch_bounds__(kSortThreads) k_bin_count_one(SortArgs s, int*
       int c;
       Real dl;
       reduce_coord<Real>(c0, one.n[t], c, dl);
-      local = local * one.nb[t] + c / one.bw[t];
+      const int b = c / one.bw[t];
+      if (t == 0) plane = c - b * one.bw[0];
+      local = local * one.nb[t] + b;
     }
-    bin[k] = gidx < s.total_points ? one.boff + local : -1;
+    key[k] = gidx < s.total_points ? one.koff + local * one.fine + (one.fine > 1 ? plane : 0) : -1;
   }
   if (any_bad) atomicOr(s.err, 1);
   unsigned peers[kSortPer];
   int got[kSortPer];
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
-    peers[k] = __match_any_sync(0xffffffffu, bin[k]);
+    peers[k] = __match_any_sync(0xffffffffu, key[k]);
     got[k] = 0;
-    if (bin[k] >= 0 && lane == __ffs(peers[k]) - 1) got[k] = atomicAdd(&bin_count[bin[k]], __popc(peers[k]));
+    if (key[k] >= 0 && lane == __ffs(peers[k]) - 1) got[k] = atomicAdd(&key_count[key[k]], __popc(peers[k]));
   }
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int first = __shfl_sync(peers[k], got[k], __ffs(peers[k]) - 1);
     const int64_t gidx = base + (int64_t)k * kSortThreads;
-    if (bin[k] >= 0) bin_rank[gidx] = make_int2(bin[k], first + __popc(peers[k] & ((1u << lane) - 1u)));
+    if (key[k] >= 0) key_rank[gidx] = make_int2(key[k], first + __popc(peers[k] & ((1u << lane) - 1u)));
   }
 }
 
 template <typename Real, int D>
-__global__ void __launch_bounds__(kSortThreads) k_scatter_one(SortArgs s, const int* __restrict__ bin_start,
-                                                              const int2* __restrict__ bin_rank, int* __restrict__ perm,
+__global__ void __launch_bounds__(kSortThreads) k_scatter_one(SortArgs s, const int* __restrict__ key_start,
+                                                              const int2* __restrict__ key_rank, int* __restrict__ perm,
                                                               uint32_t* __restrict__ local, Real* d0, Real* d1, Real* d2) {
   const int64_t base = (int64_t)blockIdx.x * (kSortThreads * kSortPer) + threadIdx.x;
   Real* dst[3] = {d0, d1, d2};
   const OneItem<D> one(s);
+  const bool whole = one.fine <= 1;   // else k_refine writes all but the index
   int2 br[kSortPer];
   double v[kSortPer][D];
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     const int64_t gidx = base + (int64_t)k * kSortThreads;
     const bool in = gidx < s.total_points;
-    br[k] = in ? bin_rank[gidx] : make_int2(-1, 0);
+    br[k] = in ? key_rank[gidx] : make_int2(-1, 0);
 #pragma unroll
-    for (int t = 0; t < D; ++t) v[k][t] = in ? one.x[(gidx - one.poff) * D + t] : 0.0;
+    for (int t = 0; t < D; ++t) v[k][t] = in && whole ? one.x[(gidx - one.poff) * D + t] : 0.0;
   }
   int pos[kSortPer];
 #pragma unroll
-  for (int k = 0; k < kSortPer; ++k) pos[k] = br[k].x >= 0 ? bin_start[br[k].x] + br[k].y : -1;
+  for (int k = 0; k < kSortPer; ++k) pos[k] = br[k].x >= 0 ? key_start[br[k].x] + br[k].y : -1;
   constexpr int bits = D == 1 ? 32 : (D == 2 ? 16 : 10);
 #pragma unroll
   for (int k = 0; k < kSortPer; ++k) {
     if (pos[k] < 0) continue;
     const int64_t gidx = base + (int64_t)k * kSortThreads;
+    perm[pos[k]] = (int)(gidx - one.poff);
+    if (!whole) continue;
     uint32_t packed = 0;
 #pragma unroll
     for (int t = 0; t < D; ++t) {
@@ -302,7 +311,6 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter_one(SortArgs s, const 
       packed |= (D == 1) ? lc : (lc << (bits * t));
       dst[t][pos[k]] = dl;
     }
-    perm[pos[k]] = (int)(gidx - one.poff);
     local[pos[k]] = packed;
   }
 }
@@ -398,9 +406,16 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* __restri
   }
 }
 
-__global__ void k_sub_count(const int* __restrict__ bin_count, int nbins, int P, int* __restrict__ sub_count) {
+__global__ void k_sub_count(SortArgs s, const int* __restrict__ key_start, int P, int* __restrict__ bin_count,
+                            int* __restrict__ bin_start, int* __restrict__ sub_count) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < nbins) sub_count[b] = (bin_count[b] + P - 1) / P;
+  if (b >= s.total_bins) return;
+  const ItemDev& it = s.items[find_item<int>(s.bin_offsets, s.n_items, b)];
+  const int key = it.key_offset + (b - it.bin_offset) * it.geom.fine;
+  const int start = key_start[key], cnt = key_start[key + it.geom.fine] - start;
+  bin_count[b] = cnt;
+  bin_start[b] = start;
+  sub_count[b] = (cnt + P - 1) / P;
 }
 
 __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const int* __restrict__ bin_start,
@@ -418,8 +433,135 @@ __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const 
     sp.start = bin_start[b] + off;
     sp.count = min(P, cnt - off);
     sp.item = item;
+    sp.dense = 0;
     subs[s0 + k] = sp;
   }
+}
+
+// The points of a pencil's subproblem (geom.fine > 1: in the order of their
+// planes, by their indices only): their records written, in runs of kRefine
+// points, ordered by cell, (l0, l1, l2), where there are as many points as
+// cells.  Neighbouring points then share cells, which interpolation turns into
+// shared-memory broadcasts (SubProblem::dense).  The scatter writes 4 bytes per point to a random place
+// instead of 20 in five arrays (32-byte sectors: 5 of them; M = 3 10^7: 1.23
+// -> 0.21 ms); the coordinates are gathered here instead, and the records go
+// out in order (1.04 ms with the sort, M = 10^6 uniform without it: 19 us).  Bitonic sort of
+// 32-bit keys (cell, slot): a step of distance 32 or less stays inside a
+// warp's 64 keys, so only the longer ones need a block barrier.
+constexpr int kRefine = 1024;
+constexpr int kRefineThreads = 256;
+constexpr int kRefinePer = kRefine / kRefineThreads;
+
+__global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProblem* __restrict__ subs,
+                                                           const int* __restrict__ num_subs, int* __restrict__ perm,
+                                                           uint32_t* __restrict__ local, float* __restrict__ d0,
+                                                           float* __restrict__ d1, float* __restrict__ d2) {
+  __shared__ uint32_t key[kRefine], loc[kRefine];
+  __shared__ int idx[kRefine];
+  __shared__ float del[3][kRefine];
+  if ((int)blockIdx.x >= *num_subs) return;
+  const SubProblem sub = subs[blockIdx.x];
+  const ItemDev& it = s.items[sub.item];
+  if (it.geom.fine <= 1) return;
+  const double* x = s.x_override ? s.x_override : it.x;
+  int n[3], bw[3];
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    n[t] = it.geom.n[t];
+    bw[t] = it.geom.bin[t];
+  }
+  int total_cells = 0;
+  for (int r0 = 0; r0 < sub.count; r0 += kRefine) {
+    const int cnt = min(kRefine, sub.count - r0), first = sub.start + r0;
+    int size = 64;
+    while (size < cnt) size *= 2;
+    // every index, then every coordinate of a thread's points in flight together
+    int j[kRefinePer];
+    double v[kRefinePer][3];
+#pragma unroll
+    for (int q = 0; q < kRefinePer; ++q) {
+      const int i = threadIdx.x + q * kRefineThreads;
+      j[q] = i < cnt ? perm[first + i] : -1;
+    }
+#pragma unroll
+    for (int q = 0; q < kRefinePer; ++q)
+#pragma unroll
+      for (int t = 0; t < 3; ++t) v[q][t] = j[q] >= 0 ? x[(int64_t)j[q] * 3 + t] : 0.0;
+#pragma unroll
+    for (int q = 0; q < kRefinePer; ++q) {
+      const int i = threadIdx.x + q * kRefineThreads;
+      if (j[q] >= 0) {
+        uint32_t packed = 0, k = 0;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          int c;
+          float dl;
+          reduce_coord<float>(isfinite(v[q][t]) ? v[q][t] : 0.0, n[t], c, dl);
+          const uint32_t lc = (uint32_t)(c % bw[t]);
+          packed |= lc << (10 * t);
+          k = t == 0 ? lc : (k << 5 | lc);   // edges of dimensions 1, 2 are below 32
+          del[t][i] = dl;
+        }
+        idx[i] = j[q];
+        loc[i] = packed;
+        key[i] = k << 10 | (uint32_t)i;
+      } else if (i < size) {
+        key[i] = 0xffffffffu;
+      }
+    }
+    __syncthreads();
+    // fewer points than cells: no run of the sort would be worth it
+    const int span = (int)((loc[cnt - 1] & 1023u) - (loc[0] & 1023u)) + 1;
+    if (cnt < span * bw[1] * bw[2]) {
+#pragma unroll
+      for (int q = 0; q < kRefinePer; ++q) {
+        const int i = threadIdx.x + q * kRefineThreads;
+        if (i >= cnt) continue;
+        local[first + i] = loc[i];
+        d0[first + i] = del[0][i];
+        d1[first + i] = del[1][i];
+        d2[first + i] = del[2][i];
+        ++total_cells;
+      }
+      __syncthreads();
+      continue;
+    }
+    for (int k = 2; k <= size; k *= 2) {
+      for (int d = k / 2; d > 0; d /= 2) {
+        for (int t = threadIdx.x; t < size / 2; t += kRefineThreads) {
+          const int a = 2 * t - (t & (d - 1));
+          const uint32_t u = key[a], v = key[a + d];
+          if ((u > v) == ((a & k) == 0)) {
+            key[a] = v;
+            key[a + d] = u;
+          }
+        }
+        // the next step is (k, d / 2) or (2 k, k)
+        if (d > 32 || (d == 1 && k > 32)) __syncthreads();
+        else __syncwarp();
+      }
+    }
+    __syncthreads();
+    int cells = 0;   // of this thread's points, those that begin a cell
+    for (int i = threadIdx.x; i < cnt; i += kRefineThreads) {
+      cells += i == 0 || key[i] >> 10 != key[i - 1] >> 10;
+      const int p = (int)(key[i] & (kRefine - 1));
+      perm[first + i] = idx[p];
+      local[first + i] = loc[p];
+      d0[first + i] = del[0][p];
+      d1[first + i] = del[1][p];
+      d2[first + i] = del[2][p];
+    }
+    total_cells += cells;
+    __syncthreads();
+  }
+  // dense: kDenseRun points per occupied cell or more
+  __shared__ int occupied;
+  if (threadIdx.x == 0) occupied = 0;
+  __syncthreads();
+  atomicAdd(&occupied, total_cells);
+  __syncthreads();
+  if (threadIdx.x == 0) subs[blockIdx.x].dense = sub.count >= kDenseRun * occupied;
 }
 
 inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -427,14 +569,14 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 }  // namespace
 
 template <typename Real>
-cudaError_t launch_bin_count(const SortArgs& s, int* bin_count, int2* bin_rank, cudaStream_t st) {
+cudaError_t launch_key_count(const SortArgs& s, int* key_count, int2* key_rank, cudaStream_t st) {
   if (s.total_points == 0) return cudaSuccess;
   const unsigned blocks = blocks_for(s.total_points, kSortThreads * kSortPer);
   switch (s.single_d) {
-    case 1: k_bin_count_one<Real, 1><<<blocks, kSortThreads, 0, st>>>(s, bin_count, bin_rank); break;
-    case 2: k_bin_count_one<Real, 2><<<blocks, kSortThreads, 0, st>>>(s, bin_count, bin_rank); break;
-    case 3: k_bin_count_one<Real, 3><<<blocks, kSortThreads, 0, st>>>(s, bin_count, bin_rank); break;
-    default: k_bin_count<Real><<<blocks, kSortThreads, 0, st>>>(s, bin_count, bin_rank);
+    case 1: k_key_count_one<Real, 1><<<blocks, kSortThreads, 0, st>>>(s, key_count, key_rank); break;
+    case 2: k_key_count_one<Real, 2><<<blocks, kSortThreads, 0, st>>>(s, key_count, key_rank); break;
+    case 3: k_key_count_one<Real, 3><<<blocks, kSortThreads, 0, st>>>(s, key_count, key_rank); break;
+    default: k_key_count<Real><<<blocks, kSortThreads, 0, st>>>(s, key_count, key_rank);
   }
   return cudaGetLastError();
 }
@@ -461,32 +603,33 @@ cudaError_t launch_scan(const int* in, int* out, int n, int* total, int* partial
 }
 
 template <typename Real>
-cudaError_t launch_scatter(const SortArgs& s, const int* bin_start, const int2* bin_rank, int* perm, uint32_t* local,
+cudaError_t launch_scatter(const SortArgs& s, const int* key_start, const int2* key_rank, int* perm, uint32_t* local,
                            Real* const* delta, cudaStream_t st) {
   if (s.total_points == 0) return cudaSuccess;
   const unsigned blocks = blocks_for(s.total_points, kSortThreads * kSortPer);
   switch (s.single_d) {
     case 1:
-      k_scatter_one<Real, 1><<<blocks, kSortThreads, 0, st>>>(s, bin_start, bin_rank, perm, local, delta[0], delta[1],
+      k_scatter_one<Real, 1><<<blocks, kSortThreads, 0, st>>>(s, key_start, key_rank, perm, local, delta[0], delta[1],
                                                               delta[2]);
       break;
     case 2:
-      k_scatter_one<Real, 2><<<blocks, kSortThreads, 0, st>>>(s, bin_start, bin_rank, perm, local, delta[0], delta[1],
+      k_scatter_one<Real, 2><<<blocks, kSortThreads, 0, st>>>(s, key_start, key_rank, perm, local, delta[0], delta[1],
                                                               delta[2]);
       break;
     case 3:
-      k_scatter_one<Real, 3><<<blocks, kSortThreads, 0, st>>>(s, bin_start, bin_rank, perm, local, delta[0], delta[1],
+      k_scatter_one<Real, 3><<<blocks, kSortThreads, 0, st>>>(s, key_start, key_rank, perm, local, delta[0], delta[1],
                                                               delta[2]);
       break;
     default:
-      k_scatter<Real><<<blocks, kSortThreads, 0, st>>>(s, bin_start, bin_rank, perm, local, delta[0], delta[1],
+      k_scatter<Real><<<blocks, kSortThreads, 0, st>>>(s, key_start, key_rank, perm, local, delta[0], delta[1],
                                                        delta[2]);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_subproblem_count(const int* bin_count, int nbins, int P, int* sub_count, cudaStream_t st) {
-  k_sub_count<<<blocks_for(nbins, 256), 256, 0, st>>>(bin_count, nbins, P, sub_count);
+cudaError_t launch_subproblem_count(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
+                                    int* sub_count, cudaStream_t st) {
+  k_sub_count<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_count);
   return cudaGetLastError();
 }
 
@@ -496,8 +639,15 @@ cudaError_t launch_subproblem_fill(const SortArgs& s, const int* bin_count, cons
   return cudaGetLastError();
 }
 
-template cudaError_t launch_bin_count<float>(const SortArgs&, int*, int2*, cudaStream_t);
-template cudaError_t launch_bin_count<double>(const SortArgs&, int*, int2*, cudaStream_t);
+cudaError_t launch_refine(const SortArgs& s, int64_t max_subs, SubProblem* subs, const int* num_subs, int* perm,
+                          uint32_t* local, float* const* delta, cudaStream_t st) {
+  if (max_subs <= 0) return cudaSuccess;
+  k_refine<<<(unsigned)max_subs, kRefineThreads, 0, st>>>(s, subs, num_subs, perm, local, delta[0], delta[1], delta[2]);
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_key_count<float>(const SortArgs&, int*, int2*, cudaStream_t);
+template cudaError_t launch_key_count<double>(const SortArgs&, int*, int2*, cudaStream_t);
 template cudaError_t launch_scatter<float>(const SortArgs&, const int*, const int2*, int*, uint32_t*, float* const*,
                                            cudaStream_t);
 template cudaError_t launch_scatter<double>(const SortArgs&, const int*, const int2*, int*, uint32_t*,
