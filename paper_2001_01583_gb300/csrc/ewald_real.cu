@@ -4,20 +4,25 @@
 // sum omits n = 0 for i = j.
 //
 // Two forms, chosen by the box:
-//   - cell list (L / r_c >= 3): the box is cut into nc^3 cells of edge
-//     h = L / nc >= r_c / 2, the ions are counting-sorted by cell, and each
-//     ion visits the 5^3 cells around its own (a partner within r_c is at
-//     most two cells away).  That is 125 h^3 ~ 15.6 r_c^3 of candidates
-//     instead of 27 r_c^3 with cells of edge r_c: the kernel issues one pair
-//     term per candidate and warp (every lane takes the same candidate, so
-//     erfc runs whenever one lane of the 32 accepts), which made the kernel
-//     issue-bound.  With r_c <= L / 3 only the minimum image of a pair can be
-//     within r_c, and it is found exactly once.  Each ion is stored as its
-//     offset from its cell's centre in FP32 (|offset| <= h / 2), so a
-//     separation (d h + o_j - o_i, |d| <= 2) carries about 1e-6 of absolute
-//     error instead of FP32's 1e-5 on box coordinates; the pair term
-//     erfc(alpha r) / r is FP32, each neighbour cell's sum is added to the
-//     ion's FP64 potential;
+//   - cell list (L / r_c >= 3): the box is cut into columns along z of edge
+//     L / ncol >= r_c / 3, each cut into fine z bins, and the ions are
+//     counting-sorted by (column, bin), so a column's ions are contiguous and
+//     nearly ordered by z.  A warp takes two ions of one column; for each of
+//     the 7 x 7 columns around it that comes within r_c it works out the z
+//     range that does and runs its lanes over the ions of that range, both
+//     partners of a lane's ion in the two halves of paired FP32 instructions.
+//     47% of the candidates are partners; of the 125 cells of edge r_c / 2
+//     around an ion, a thread per ion, 23% were, and every candidate ran the
+//     whole pair term because one lane of 32 accepted it.  393216 ions,
+//     r_c = 10, about 4000 partners each, with forces: 12.8 -> 4.7 ms.  It is
+//     bound by issue (70 instructions per 64 candidates, 60% of the slots) and
+//     the FP32 pipe (25 of them paired operations of two cycles).
+//     With r_c <= L / 3 only the minimum image of a pair can be within r_c,
+//     and it is found exactly once.  Lengths are in units of L.  An ion's x
+//     and y are FP32 offsets from its column's axis, its z the sum of a
+//     multiple of 2^-10 and an FP32 remainder, so that separations carry an
+//     error of about 1e-9 L and neither box coordinates nor periodic shifts
+//     are rounded; pair terms and a lane's sums are FP32;
 //   - all pairs (smaller boxes): the minimum image of every pair plus the 26
 //     shifts by L, all in FP64, which is the definition itself (r_c < L).
 // The energy 1/2 sum_i q_i phi_i is reduced in FP64 in a fixed order (block
@@ -32,12 +37,45 @@
 
 #include "gbnfft.h"
 #include "kernels.h"
+#include "warp.cuh"
 
 namespace gbnfft {
 namespace {
 
 constexpr int kRsThreads = 256;
-constexpr int kRsReach = 2;   // neighbour cells per side (cell edge >= r_c / kRsReach)
+constexpr int kRsReach = 3;     // neighbour columns per side (column edge >= r_c / kRsReach)
+constexpr int kRsColumns = (2 * kRsReach + 1) * (2 * kRsReach + 1);
+constexpr int kRsIons = 8;      // ions a warp takes, two at a time
+constexpr double kRsGrid = 1024.0;
+
+// (v, v), kept in its registers (the compiler rebuilt constant pairs in the loop).
+__device__ __forceinline__ Pair pinned_pair(float v) {
+  Pair p;
+  asm volatile("mov.b64 %0, {%1, %1};" : "=l"(p) : "f"(v));
+  return p;
+}
+// The hardware's 2^x, 1 / x and 1 / sqrt(x) (a few ulp) in both halves.
+__device__ __forceinline__ Pair pair_exp2(Pair p) {
+  const float2 v = halves(p);
+  float a, b;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(v.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(v.y));
+  return pair(a, b);
+}
+__device__ __forceinline__ Pair pair_rcp(Pair p) {
+  const float2 v = halves(p);
+  float a, b;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(v.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(v.y));
+  return pair(a, b);
+}
+__device__ __forceinline__ Pair pair_rsqrt(Pair p) {
+  const float2 v = halves(p);
+  float a, b;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(v.x));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(v.y));
+  return pair(a, b);
+}
 
 __device__ __forceinline__ double warp_sum_f64(double v) {
 #pragma unroll
@@ -59,105 +97,204 @@ __device__ __forceinline__ void block_partial(double v, double* partial) {
   }
 }
 
-// Cell of each ion (coordinates reduced into [0, L)) and its rank in the cell.
-__global__ void k_rs_count(int64_t n, const double* __restrict__ r, double L, int nc, int* __restrict__ count,
+// Fraction of the box edge in [0, 1), and its cell of n.
+__device__ __forceinline__ double rs_fraction(double r, double L) {
+  const double u = r / L;
+  const double s = u - floor(u);
+  return s < 1.0 ? s : 0.0;
+}
+__device__ __forceinline__ int rs_cell(double s, int n) { return min((int)(s * n), n - 1); }
+
+// (Column, z bin) of each ion and its rank there.
+__global__ void k_rs_count(int64_t n, const double* __restrict__ r, double L, int ncol, int nz, int* __restrict__ count,
                            int2* __restrict__ cell_rank) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int c[3];
-  for (int t = 0; t < 3; ++t) {
-    const double u = r[i * 3 + t] / L;
-    const double s = (u - floor(u)) * nc;
-    int ct = (int)floor(s);
-    c[t] = ct < 0 ? 0 : (ct >= nc ? nc - 1 : ct);
-  }
-  const int cell = (c[0] * nc + c[1]) * nc + c[2];
+  const int cx = rs_cell(rs_fraction(r[i * 3], L), ncol), cy = rs_cell(rs_fraction(r[i * 3 + 1], L), ncol);
+  const int cell = (cx * ncol + cy) * nz + rs_cell(rs_fraction(r[i * 3 + 2], L), nz);
   cell_rank[i] = make_int2(cell, atomicAdd(&count[cell], 1));
 }
 
-// Sorted record: offset from the cell centre (FP32) and the charge.
-__global__ void k_rs_scatter(int64_t n, const double* __restrict__ r, const double* __restrict__ q, double L, int nc,
-                             const int* __restrict__ start, const int2* __restrict__ cell_rank,
-                             float4* __restrict__ rec, int* __restrict__ rec_cell, int* __restrict__ rec_idx) {
+// Sorted records: (x, y offsets from the column's axis, z in two parts), the
+// charge and the column.
+__global__ void k_rs_scatter(int64_t n, const double* __restrict__ r, const double* __restrict__ q, double L, int ncol,
+                             int nz, const int* __restrict__ start, const int2* __restrict__ cell_rank,
+                             float4* __restrict__ rec, float* __restrict__ rec_q, int* __restrict__ rec_col,
+                             int* __restrict__ rec_idx) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int2 cr = cell_rank[i];
-  const int cz = cr.x % nc, cy = (cr.x / nc) % nc, cx = cr.x / (nc * nc);
-  const int cc[3] = {cx, cy, cz};
-  const double h = L / nc;
-  float o[3];
-  for (int t = 0; t < 3; ++t) {
-    const double u = r[i * 3 + t] / L;
-    const double pos = (u - floor(u)) * L;   // in [0, L]
-    o[t] = (float)(pos - (cc[t] + 0.5) * h);
-  }
+  const int col = cr.x / nz;
+  const double sx = rs_fraction(r[i * 3], L), sy = rs_fraction(r[i * 3 + 1], L), sz = rs_fraction(r[i * 3 + 2], L);
+  const double zh = floor(sz * kRsGrid) / kRsGrid;
   const int p = start[cr.x] + cr.y;
-  rec[p] = make_float4(o[0], o[1], o[2], (float)q[i]);
-  rec_cell[p] = cr.x;
+  rec[p] = make_float4((float)(sx - (col / ncol + 0.5) / ncol), (float)(sy - (col % ncol + 0.5) / ncol), (float)zh,
+                       (float)(sz - zh));
+  // an ion without a position takes no part
+  const bool placed = isfinite(r[i * 3]) && isfinite(r[i * 3 + 1]) && isfinite(r[i * 3 + 2]);
+  rec_q[p] = placed ? (float)q[i] : 0.f;
+  rec_col[p] = col;
   if (rec_idx) rec_idx[p] = (int)i;
 }
 
-constexpr float kTwoOverSqrtPiF = 1.1283791670955126f;
 constexpr double kTwoOverSqrtPi = 1.1283791670955126;
 
-// Potential of each sorted ion from the 27 cells around its own; block
-// partials of q_i phi_i.  FORCES: also the ion's force, written to its
-// original index (F: n x 3 doubles).
+// erfc(x) e^(x^2) for x >= 0 as t P(t), t = 1 / (1 + 0.42 x): P is the
+// least relative error polynomial of degree 7 over x in [0, 6.5] (Chebyshev
+// fit with iterated weights): 4e-8, 1e-7 with FP32 rounding.  Beyond, e^(-x^2)
+// is below 1e-18.
+constexpr float kErfcScale = 0.42f;
+
+struct RsParams {
+  int n, ncol, nz;
+  float rc2, near;  // (r_c / L)^2, r_c / (4 L)
+  float alpha;      // alpha L
+  float escale;     // -(alpha L)^2 log2(e)
+  float c2;         // 2 alpha L / sqrt(pi)
+  double phi_scale, f_scale;   // 1 / L, 1 / L^2
+};
+
+// A range of ions in a column: the offsets of its axis, the z shift of its image.
+struct RsRange {
+  int begin, end;
+  float dx, dy, dz;
+};
+
+// Potential (and force) of each sorted ion; block partials of q_i phi_i.
+// FORCES: also the ion's force, written to its original index (F: n x 3).
 template <bool FORCES>
-__global__ void __launch_bounds__(kRsThreads) k_rs_cells(int n, int nc, float h, float rc2, float alpha,
-                                                         const float4* __restrict__ rec,
-                                                         const int* __restrict__ rec_cell,
-                                                         const int* __restrict__ start, double* __restrict__ partial,
-                                                         const int* __restrict__ rec_idx, double* __restrict__ F) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kRsThreads, 4) k_rs_columns(RsParams P, const float4* __restrict__ rec,
+                                                           const float* __restrict__ rec_q,
+                                                           const int* __restrict__ rec_col,
+                                                           const int* __restrict__ start, double* __restrict__ partial,
+                                                           const int* __restrict__ rec_idx, double* __restrict__ F) {
+  __shared__ RsRange ranges[kRsThreads / 32][2 * kRsColumns];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  RsRange* mine = ranges[warp];
+  const int first = (blockIdx.x * (kRsThreads / 32) + warp) * kRsIons, last = min(P.n, first + kRsIons);
+  const float inv = 1.0f / (float)P.ncol, half = 0.5f * inv;
+  constexpr float kErfc[8] = {0.236731262f, 0.240897215f,  0.187104512f,  0.292422239f,
+                              -0.17306915f, 0.48496216f,   -0.345052719f, 0.0760044978f};
+  // added to every squared distance, so that the pair term of an ion with
+  // itself (masked) stays finite; far below what the records resolve
+  constexpr float tiny = 1e-20f;
+  Pair cf[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) cf[c] = pinned_pair(kErfc[c]);
+  const Pair ps = pinned_pair(kErfcScale * P.alpha), one = pinned_pair(1.f), tn = pinned_pair(tiny);
+  const Pair es = pinned_pair(P.escale), c2 = pinned_pair(P.c2);
+  const float rc2 = P.rc2;
   double e = 0.0;
-  if (i < n) {
-    const float4 pi = rec[i];
-    const int cell = rec_cell[i];
-    const int cz = cell % nc, cy = (cell / nc) % nc, cx = cell / (nc * nc);
-    double phi = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
-    const float c2 = kTwoOverSqrtPiF * alpha, a2 = alpha * alpha;
-    for (int dx = -kRsReach; dx <= kRsReach; ++dx) {
-      const int x = cx + dx < 0 ? cx + dx + nc : (cx + dx >= nc ? cx + dx - nc : cx + dx);
-      for (int dy = -kRsReach; dy <= kRsReach; ++dy) {
-        const int y = cy + dy < 0 ? cy + dy + nc : (cy + dy >= nc ? cy + dy - nc : cy + dy);
-        for (int dz = -kRsReach; dz <= kRsReach; ++dz) {
-          const int z = cz + dz < 0 ? cz + dz + nc : (cz + dz >= nc ? cz + dz - nc : cz + dz);
-          const int nb = (x * nc + y) * nc + z;
-          const float sx = dx * h - pi.x, sy = dy * h - pi.y, sz = dz * h - pi.z;
-          float acc = 0.0f, ax = 0.0f, ay = 0.0f, az = 0.0f;
-          for (int j = start[nb]; j < start[nb + 1]; ++j) {
-            const float4 pj = rec[j];
-            const float rx = pj.x + sx, ry = pj.y + sy, rz = pj.z + sz;   // r_j - r_i
-            const float d2 = rx * rx + ry * ry + rz * rz;
-            if (d2 < rc2 && d2 > 0.0f) {
-              const float rinv = rsqrtf(d2);
-              const float ec = erfcf(alpha * d2 * rinv) * rinv;
-              acc += pj.w * ec;
-              if (FORCES) {
-                const float g = pj.w * (ec + c2 * __expf(-a2 * d2)) * rinv * rinv;
-                ax -= g * rx;
-                ay -= g * ry;
-                az -= g * rz;
-              }
-            }
-          }
-          phi += (double)acc;
-          if (FORCES) {
-            fx += (double)ax;
-            fy += (double)ay;
-            fz += (double)az;
-          }
+  for (int i = first; i < last;) {
+    // two ions of one column, or one (then both halves hold it)
+    const int col = rec_col[i];
+    const float4 pa = rec[i];
+    float4 pb = rec[min(i + 1, P.n - 1)];
+    const float za = pa.z + pa.w;
+    float zb = pb.z + pb.w;
+    // close in z as well: their common range then wraps on one side at most
+    const bool two = i + 1 < last && rec_col[i + 1] == col && fabsf(zb - za) <= P.near;
+    if (!two) {
+      pb = pa;
+      zb = za;
+    }
+    const int cx = col / P.ncol, cy = col - cx * P.ncol;
+    // the ranges of the columns around: up to two each (the z period)
+    int count = 0;
+    __syncwarp();
+    for (int t0 = 0; t0 < kRsColumns; t0 += 32) {
+      const int t = t0 + lane;
+      const int ix = t / (2 * kRsReach + 1) - kRsReach, iy = t % (2 * kRsReach + 1) - kRsReach;
+      RsRange rg;
+      rg.dx = (float)ix * inv;
+      rg.dy = (float)iy * inv;
+      rg.dz = 0.f;
+      const float mx = fmaxf(fminf(fabsf(rg.dx - pa.x), fabsf(rg.dx - pb.x)) - half, 0.f);
+      const float my = fmaxf(fminf(fabsf(rg.dy - pa.y), fabsf(rg.dy - pb.y)) - half, 0.f);
+      const float left = P.rc2 * 1.00001f - mx * mx - my * my;
+      int b0 = 0, b1 = -1, w0 = 0, w1 = -1;   // bins in the box, and of the image above or below
+      float wz = 0.f;
+      int base = 0;
+      if (t < kRsColumns && left > 0.f) {
+        const int x = cx + ix < 0 ? cx + ix + P.ncol : (cx + ix >= P.ncol ? cx + ix - P.ncol : cx + ix);
+        const int y = cy + iy < 0 ? cy + iy + P.ncol : (cy + iy >= P.ncol ? cy + iy - P.ncol : cy + iy);
+        base = (x * P.ncol + y) * P.nz;
+        const float reach = sqrtf(left);
+        b0 = (int)floorf((fminf(za, zb) - reach) * (float)P.nz - 1e-3f);
+        b1 = (int)floorf((fmaxf(za, zb) + reach) * (float)P.nz + 1e-3f);
+        if (b0 < 0) {
+          w0 = b0 + P.nz, w1 = P.nz - 1, wz = -1.f;
+          b0 = 0;
+        } else if (b1 >= P.nz) {
+          w0 = 0, w1 = b1 - P.nz, wz = 1.f;
+          b1 = P.nz - 1;
         }
       }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int lo = k ? w0 : b0, hi = k ? w1 : b1;
+        bool some = lo <= hi;
+        if (some) {
+          rg.begin = start[base + lo];
+          rg.end = start[base + hi + 1];
+          if (k) rg.dz = wz;
+          some = rg.begin < rg.end;
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, some);
+        if (some) mine[count + __popc(mask & ((1u << lane) - 1u))] = rg;
+        count += __popc(mask);
+      }
     }
-    e = (double)pi.w * phi;
-    if (FORCES) {
-      const int64_t o = (int64_t)rec_idx[i] * 3;
-      F[o] = (double)pi.w * fx;
-      F[o + 1] = (double)pi.w * fy;
-      F[o + 2] = (double)pi.w * fz;
+    __syncwarp();
+    Pair phi = 0, fx = 0, fy = 0, fz = 0;
+    for (int k = 0; k < count; ++k) {
+      const RsRange rg = mine[k];
+      const float sxa = rg.dx - pa.x, sxb = rg.dx - pb.x, sya = rg.dy - pa.y, syb = rg.dy - pb.y;
+      // a range's sums on their own first: shorter FP32 sums
+      Pair rphi = 0, rfx = 0, rfy = 0, rfz = 0;
+      const float sha = rg.dz - pa.z, shb = rg.dz - pb.z, sla = -pa.w, slb = -pb.w;
+#pragma unroll 2
+      for (int j0 = rg.begin; j0 < rg.end; j0 += 32) {
+        const int j = min(j0 + lane, rg.end - 1);
+        const float4 rj = __ldg(rec + j);
+        const float qj = j0 + lane < rg.end ? __ldg(rec_q + j) : 0.f;
+        // single adds: a paired one would first copy rj into both halves
+        const Pair X = pair(rj.x + sxa, rj.x + sxb), Y = pair(rj.y + sya, rj.y + syb);
+        const Pair Z = pair_add(pair(rj.z + sha, rj.z + shb), pair(rj.w + sla, rj.w + slb));
+        const Pair d2p = pair_fma(Z, Z, pair_fma(Y, Y, pair_fma(X, X, tn)));
+        const float2 d2 = halves(d2p);
+        const float qa = d2.x < rc2 && d2.x > tiny ? qj : 0.f, qb = d2.y < rc2 && d2.y > tiny ? qj : 0.f;
+        const Pair rinv = pair_rsqrt(d2p);
+        const Pair t = pair_rcp(pair_fma(pair_mul(d2p, rinv), ps, one)), ee = pair_exp2(pair_mul(d2p, es));
+        Pair w = cf[7];
+#pragma unroll
+        for (int c = 6; c >= 0; --c) w = pair_fma(w, t, cf[c]);
+        const Pair q2 = pair(qa, qb);
+        const Pair ec = pair_mul(pair_mul(pair_mul(w, t), ee), rinv);   // erfc(alpha r) / r
+        rphi = pair_fma(q2, ec, rphi);
+        if (FORCES) {
+          const Pair g = pair_mul(pair_mul(pair_fma(ee, c2, ec), pair_mul(rinv, rinv)), q2);
+          rfx = pair_fma(g, X, rfx);
+          rfy = pair_fma(g, Y, rfy);
+          rfz = pair_fma(g, Z, rfz);
+        }
+      }
+      phi = pair_add(phi, rphi);
+      fx = pair_add(fx, rfx);
+      fy = pair_add(fy, rfy);
+      fz = pair_add(fz, rfz);
     }
+    // over the warp: lane l gets value l >> 2 of (phi, f) of the first ion, then of the second
+    const float2 p2 = halves(phi), x2 = halves(fx), y2 = halves(fy), z2 = halves(fz);
+    const float v[8] = {p2.x, x2.x, y2.x, z2.x, p2.y, x2.y, y2.y, z2.y};
+    const float sum = butterfly8(v, lane);
+    const int which = lane >> 4, comp = (lane >> 2) & 3;
+    if ((lane & 3) == 0 && (which == 0 || two)) {
+      const double qi = (double)rec_q[i + which];
+      if (comp == 0) e += qi * (double)sum * P.phi_scale;
+      else if (FORCES) F[(int64_t)rec_idx[i + which] * 3 + comp - 1] = -qi * (double)sum * P.f_scale;
+    }
+    i += two ? 2 : 1;
   }
   block_partial(e, partial);
 }
@@ -227,20 +364,23 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
   *energy = 0.0;
   if (n == 0) return NFFT_OK;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // cells of edge L / nc >= rcut / kRsReach (at least 2 kRsReach + 1 of them
-  // per side, so the neighbour cells are distinct); L / rcut < 3: all pairs
-  const int nc = (int)std::floor(L / rcut) < 3 ? 1 : std::min((int)std::floor(kRsReach * L / rcut), 256);
-  if (nc == 1 && n > 65536) return NFFT_ERR_UNSUPPORTED;   // the all-pairs form is O(n^2)
+  // columns of edge L / ncol >= rcut / kRsReach (at least 9 per side, so the
+  // 7 x 7 around one are distinct), z bins a quarter of that; L / rcut < 3: all pairs
+  const bool cells_form = std::floor(L / rcut) >= 3;
+  const int ncol = cells_form ? std::min((int)std::floor(kRsReach * L / rcut), 128) : 1, nz = 4 * ncol;
+  if (!cells_form && n > 65536) return NFFT_ERR_UNSUPPORTED;   // the all-pairs form is O(n^2)
   const int ni = (int)n;
   const int blocks = (ni + kRsThreads - 1) / kRsThreads;
-  const int cells = nc * nc * nc;
-  // scratch: partials (blocks + 1), and for the cell list counts, starts,
-  // scan scratch, (cell, rank), records, record cells and record indices
-  size_t bytes = sizeof(double) * (size_t)(blocks + 1);
-  if (nc > 1) {
-    bytes += sizeof(int) * (size_t)(2 * cells + 2) + sizeof(int2) * (size_t)n + sizeof(float4) * (size_t)n +
-             sizeof(int) * (size_t)n + sizeof(int) * (size_t)scan_partials_needed(cells + 1) +
-             (F_dev ? sizeof(int) * (size_t)n : 0) + 64;
+  constexpr int per_block = kRsThreads / 32 * kRsIons;
+  const int parts = cells_form ? (ni + per_block - 1) / per_block : blocks;
+  const int cells = ncol * ncol * nz;
+  // scratch: partials and the total, and for the cell list records, charges,
+  // (cell, rank), columns, counts, starts, scan scratch and record indices
+  size_t bytes = sizeof(double) * (size_t)(parts + 1);
+  if (cells_form) {
+    bytes += 16 + (sizeof(float4) + sizeof(int2) + sizeof(float) + sizeof(int)) * ((size_t)n + 1) +
+             sizeof(int) * ((size_t)(2 * cells + 2) + (size_t)scan_partials_needed(cells + 1)) +
+             (F_dev ? sizeof(int) * (size_t)n : 0);
   }
   char* buf = nullptr;
   if (cudaMalloc(&buf, bytes) != cudaSuccess) {
@@ -252,29 +392,39 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
     if (e != cudaSuccess && status == NFFT_OK) status = NFFT_ERR_CUDA;
   };
   double* partial = reinterpret_cast<double*>(buf);
-  double* total = partial + blocks;
-  if (nc > 1) {
-    char* p = buf + sizeof(double) * (size_t)(blocks + 1);
+  double* total = partial + parts;
+  if (cells_form) {
+    char* p = buf + sizeof(double) * (size_t)(parts + 1);
     float4* rec = reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(p) + 15) & ~(uintptr_t)15);
-    int* rec_cell = reinterpret_cast<int*>(rec + n);
-    int2* cell_rank = reinterpret_cast<int2*>(rec_cell + n + (n & 1));
-    int* count = reinterpret_cast<int*>(cell_rank + n);
+    int2* cell_rank = reinterpret_cast<int2*>(rec + n);
+    float* rec_q = reinterpret_cast<float*>(cell_rank + n);
+    int* rec_col = reinterpret_cast<int*>(rec_q + n);
+    int* count = rec_col + n;
     int* start = count + cells + 1;
     int* scan_scratch = start + cells + 1;
     int* rec_idx = F_dev ? scan_scratch + scan_partials_needed(cells + 1) : nullptr;
     ck(cudaMemsetAsync(count, 0, sizeof(int) * (size_t)(cells + 1), st));
-    k_rs_count<<<blocks, kRsThreads, 0, st>>>(n, r_dev, L, nc, count, cell_rank);
+    k_rs_count<<<blocks, kRsThreads, 0, st>>>(n, r_dev, L, ncol, nz, count, cell_rank);
     ck(cudaGetLastError());
     ck(launch_scan(count, start, cells + 1, nullptr, scan_scratch, st));   // start[cells] = n
-    k_rs_scatter<<<blocks, kRsThreads, 0, st>>>(n, r_dev, q_dev, L, nc, start, cell_rank, rec, rec_cell, rec_idx);
+    k_rs_scatter<<<blocks, kRsThreads, 0, st>>>(n, r_dev, q_dev, L, ncol, nz, start, cell_rank, rec, rec_q, rec_col,
+                                                rec_idx);
     ck(cudaGetLastError());
-    const double h = L / nc;
+    RsParams P;
+    P.n = ni;
+    P.ncol = ncol;
+    P.nz = nz;
+    P.rc2 = (float)(rcut / L * (rcut / L));
+    P.near = (float)(0.25 * rcut / L);
+    P.alpha = (float)(alpha * L);
+    P.escale = (float)(-alpha * L * alpha * L * 1.4426950408889634);
+    P.c2 = (float)(kTwoOverSqrtPi * alpha * L);
+    P.phi_scale = 1.0 / L;
+    P.f_scale = 1.0 / (L * L);
     if (F_dev)
-      k_rs_cells<true><<<blocks, kRsThreads, 0, st>>>(ni, nc, (float)h, (float)(rcut * rcut), (float)alpha, rec,
-                                                      rec_cell, start, partial, rec_idx, F_dev);
+      k_rs_columns<true><<<parts, kRsThreads, 0, st>>>(P, rec, rec_q, rec_col, start, partial, rec_idx, F_dev);
     else
-      k_rs_cells<false><<<blocks, kRsThreads, 0, st>>>(ni, nc, (float)h, (float)(rcut * rcut), (float)alpha, rec,
-                                                       rec_cell, start, partial, nullptr, nullptr);
+      k_rs_columns<false><<<parts, kRsThreads, 0, st>>>(P, rec, rec_q, rec_col, start, partial, nullptr, nullptr);
     ck(cudaGetLastError());
   } else {
     if (F_dev)
@@ -283,7 +433,7 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
       k_rs_pairs<false><<<blocks, kRsThreads, 0, st>>>(ni, r_dev, q_dev, L, rcut, alpha, partial, nullptr);
     ck(cudaGetLastError());
   }
-  k_rs_total<<<1, kRsThreads, 0, st>>>(partial, blocks, 0.5, total);
+  k_rs_total<<<1, kRsThreads, 0, st>>>(partial, parts, 0.5, total);
   ck(cudaGetLastError());
   double host = 0.0;
   ck(cudaMemcpyAsync(&host, total, sizeof(double), cudaMemcpyDeviceToHost, st));

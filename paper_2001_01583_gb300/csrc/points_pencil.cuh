@@ -160,26 +160,6 @@ struct PencilFetch {
   }
 };
 
-// Two neighbouring floats in one 64-bit register pair (a window assembled from
-// scalars as float2 was copied into aligned pairs for every point: 37 moves).
-using Pair = unsigned long long;
-__device__ __forceinline__ Pair pair(float lo, float hi) {
-  Pair p;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(lo), "f"(hi));
-  return p;
-}
-__device__ __forceinline__ float2 halves(Pair p) {
-  float2 v;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
-}
-// a b + c in each half, one rounding each
-__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c) {
-  Pair d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-
 // W floats (W even) from a 16-byte aligned shared address, as pairs.
 template <int W>
 __device__ __forceinline__ void lds_pairs(uint32_t a, Pair* w) {

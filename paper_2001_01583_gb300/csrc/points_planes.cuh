@@ -27,6 +27,7 @@
 #pragma once
 
 #include "points_tiled.cuh"
+#include "warp.cuh"
 
 namespace gbnfft {
 
@@ -695,37 +696,6 @@ __global__ void __launch_bounds__(32 * NW) k_spread_planes(PointKernelArgs<Real>
       __syncthreads();
     }
   }
-}
-
-// The 4 points' 8 real values of a warp pass (v[2g], v[2g + 1]: this lane's
-// share of point g), reduced over the warp at once by a transposed
-// butterfly (9 shuffles): after the exchanges over lane bits 4, 3 and 2 each
-// lane keeps one value, and bits 1 and 0 finish its sum.  Lane l returns the
-// sum of value l >> 2.
-__device__ __forceinline__ float butterfly8(const float* v, int lane) {
-  const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
-  float a4[4], a2[2];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float send = b4 ? v[j] : v[4 + j];
-    const float keep = b4 ? v[4 + j] : v[j];
-    a4[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float send = b3 ? a4[j] : a4[2 + j];
-    const float keep = b3 ? a4[2 + j] : a4[j];
-    a2[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  float a1;
-  {
-    const float send = b2 ? a2[0] : a2[1];
-    const float keep = b2 ? a2[1] : a2[0];
-    a1 = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
-  a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
-  return a1;
 }
 
 // butterfly8 of points p0 .. p0 + 3: lane 8g writes point p0 + g to its place in the caller's order.
