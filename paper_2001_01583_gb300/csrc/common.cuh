@@ -203,22 +203,6 @@ __device__ __forceinline__ void window_taps(const WindowDev& win, int t, double 
 }
 
 // One of them, tap k (kernels whose lanes take different taps).
-__device__ __forceinline__ float window_tap(const WindowDev& win, int t, float delta, int k, int taps) {
-  const bool mirror = k >= taps / 2;
-  const float4* c = reinterpret_cast<const float4*>(win.polyf[t]) + (mirror ? taps - 1 - k : k) * (kPolyF / 2);
-  const float x = fmaf(2.0f, delta, -1.0f);
-  const float s = x * x;
-  float2 p;
-#pragma unroll
-  for (int q = kPolyF / 2 - 1; q >= 0; --q) {
-    const float4 v = __ldg(c + q);
-    if (q == kPolyF / 2 - 1) p = make_float2(v.z, v.w);
-    else p = cmad(p, s, make_float2(v.z, v.w));
-    p = cmad(p, s, make_float2(v.x, v.y));
-  }
-  if (win.kind != 0 && delta == 0.0f && k == taps - 1) return 0.0f;
-  return fmaf(mirror ? -x : x, p.y, p.x);
-}
 __device__ __forceinline__ double window_tap(const WindowDev& win, int t, double delta, int k, int taps) {
   const bool mirror = k >= taps / 2;
   const double2* c = win.polyd[t] + (mirror ? taps - 1 - k : k) * kPolyD;

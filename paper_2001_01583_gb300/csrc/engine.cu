@@ -432,6 +432,13 @@ int Engine::build_layout() {
   points_set = false;
   const int nitems = (int)specs.size();
   max_sub = max_sub_opt > 0 ? max_sub_opt : 1024;
+  // few points: subproblems small enough for two per SM (N = 256, M = 1024 in
+  // 1-D, FP64, one bin of 512 cells: spreading 72 -> 16 us, interpolation 51 -> 12)
+  if (max_sub_opt == 0) {
+    int64_t total = 0;
+    for (const auto& s : specs) total += s.M;
+    max_sub = (int)std::min<int64_t>(1024, std::max<int64_t>(32, total / (2 * (int64_t)num_sms)));
+  }
   const size_t budget = smem_optin < kSmemBudget ? smem_optin : kSmemBudget;
 
   struct Choice {
@@ -549,7 +556,7 @@ int Engine::build_layout() {
       auto pick = [&](int opt, double per_cell) {
         if (opt < 0) return 0;
         if (opt > 0) return opt;
-        return std::max(1, std::min((int)std::ceil(per_cell * cells / foot), max_sub));
+        return std::max(1, std::min((int)std::ceil(per_cell * cells / foot), max_sub_opt > 0 ? max_sub : 1024));
       };
       c.sparse = pick(sparse_opt, 2.0);
       c.sparse_interp = pick(sparse_interp_opt, 5.0);
@@ -756,6 +763,7 @@ int Engine::build_layout() {
   TRY(alloc_dev(d_bin_offsets, sizeof(int) * (nitems + 1), device_bytes));
   const size_t K = (size_t)std::max(total_keys, 1);
   TRY(alloc_dev(key_count, sizeof(int) * K, device_bytes));
+  CK(cudaMemset(key_count, 0, sizeof(int) * K));
   TRY(alloc_dev(key_start, sizeof(int) * (K + 1), device_bytes));
   TRY(alloc_dev(bin_count, sizeof(int) * B, device_bytes));
   TRY(alloc_dev(bin_start, sizeof(int) * B, device_bytes));
@@ -1300,16 +1308,14 @@ int Engine::set_points_impl(const double* x_override) {
   s.single_d = items.size() == 1 ? items[0].geom.d : 0;
   EventPair ev{};
   TRY(stage_begin(NFFT_STAGE_SORT, &ev));
-  CK(cudaMemsetAsync(key_count, 0, sizeof(int) * (size_t)std::max(total_keys, 1), stream));
+  // (key_count is zero: the layout clears it, and so does every scan)
   CK(launch_key_count<Real>(s, key_count, key_rank, stream));
-  // key count, scatter, subproblem count and fill, two scans
-  kernel_launches += (s.total_points > 0 ? 4 : 2) + scan_launches(total_keys) + scan_launches(total_bins);
-  CK(launch_scan(key_count, key_start, total_keys, key_start + total_keys, scan_partials, stream));
+  kernel_launches += (s.total_points > 0 ? 2 : 0) + scan_launches(total_keys) + subproblem_launches(total_bins);
+  CK(launch_scan(key_count, key_start, total_keys, key_start + total_keys, scan_partials, true, stream));
   Real* d[3] = {static_cast<Real*>(delta[0]), static_cast<Real*>(delta[1]), static_cast<Real*>(delta[2])};
   CK(launch_scatter<Real>(s, key_start, key_rank, perm, local, d, stream));
-  CK(launch_subproblem_count(s, key_start, max_sub, bin_count, bin_start, sub_count, stream));
-  CK(launch_scan(sub_count, sub_start, total_bins, num_subs, scan_partials, stream));
-  CK(launch_subproblem_fill(s, bin_count, bin_start, sub_start, max_sub, subs, stream));
+  CK(launch_subproblems(s, key_start, max_sub, bin_count, bin_start, sub_count, sub_start, num_subs, scan_partials,
+                        subs, stream));
   if constexpr (sizeof(Real) == 4) {
     bool pencils = false;
     for (const auto& kc : kclasses) pencils = pencils || kc.pencil;

@@ -406,7 +406,7 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
     ck(cudaMemsetAsync(count, 0, sizeof(int) * (size_t)(cells + 1), st));
     k_rs_count<<<blocks, kRsThreads, 0, st>>>(n, r_dev, L, ncol, nz, count, cell_rank);
     ck(cudaGetLastError());
-    ck(launch_scan(count, start, cells + 1, nullptr, scan_scratch, st));   // start[cells] = n
+    ck(launch_scan(count, start, cells + 1, nullptr, scan_scratch, false, st));   // start[cells] = n
     k_rs_scatter<<<blocks, kRsThreads, 0, st>>>(n, r_dev, q_dev, L, ncol, nz, start, cell_rank, rec, rec_q, rec_col,
                                                 rec_idx);
     ck(cudaGetLastError());

@@ -34,19 +34,19 @@ cudaError_t launch_key_count(const SortArgs& s, int* key_count, int2* key_rank, 
 // scan_partials_needed(n) ints of device scratch.  scan_launches(n) kernels.
 int scan_partials_needed(int n);
 int scan_launches(int n);
-cudaError_t launch_scan(const int* in, int* out, int n, int* total, int* partials, cudaStream_t st);
+// clear: the input is left zero.
+cudaError_t launch_scan(int* in, int* out, int n, int* total, int* partials, bool clear, cudaStream_t st);
 // Write every point to its sorted slot: perm (index within its item), packed in-bin offsets, deltas.
 template <typename Real>
 cudaError_t launch_scatter(const SortArgs& s, const int* key_start, const int2* key_rank, int* perm, uint32_t* local,
                            Real* const* delta, cudaStream_t st);
-// Points, first sorted position and subproblems (ceil(count / P)) of every
-// global bin from its keys (key_start: their exclusive scan, one past the end
-// too), then the subproblems' records.
-cudaError_t launch_subproblem_count(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
-                                    int* sub_count, cudaStream_t st);
-cudaError_t launch_subproblem_fill(const SortArgs& s, const int* bin_count, const int* bin_start, const int* sub_start,
-                                   int P, SubProblem* subs, cudaStream_t st);
-
+// Points, first sorted position and first subproblem (ceil(count / P) each) of
+// every global bin from its keys (key_start: their exclusive scan, one past the
+// end too), and the subproblems' records.  subproblem_launches(bins) kernels.
+int subproblem_launches(int nbins);
+cudaError_t launch_subproblems(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
+                               int* sub_count, int* sub_start, int* num_subs, int* partials, SubProblem* subs,
+                               cudaStream_t st);
 // Pencil items (GridGeom::fine > 1): the points of every subproblem ordered by
 // cell and their records written (the scatter writes their indices only).
 cudaError_t launch_refine(const SortArgs& s, int64_t max_subs, SubProblem* subs, const int* num_subs, int* perm,

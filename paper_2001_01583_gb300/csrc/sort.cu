@@ -318,8 +318,9 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter_one(SortArgs s, const 
 // Exclusive scan of n ints with one block of 1024 threads: each thread scans a
 // contiguous chunk sequentially, the chunk totals are scanned in shared memory.
 // Used for the per-tile partial sums of the multi-block scan below.
-__global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ in, int* __restrict__ out, int n,
-                                                int* __restrict__ total) {
+// clear: the input is left zero (the sort's counts, for the next call).
+__global__ void __launch_bounds__(1024) k_scan(int* __restrict__ in, int* __restrict__ out, int n,
+                                                int* __restrict__ total, bool clear) {
   __shared__ int part[1024];
   const int T = blockDim.x;
   const int chunk = (n + T - 1) / T;
@@ -340,6 +341,7 @@ __global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ in, int* 
   for (int i = lo; i < hi; ++i) {
     const int v = in[i];
     out[i] = run;
+    if (clear) in[i] = 0;
     run += v;
   }
   if (total && threadIdx.x == T - 1) *total = part[T - 1];
@@ -388,8 +390,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int* __restr
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* __restrict__ in, int* __restrict__ out, int n,
-                                                              const int* __restrict__ offsets) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(int* __restrict__ in, int* __restrict__ out, int n,
+                                                              const int* __restrict__ offsets, bool clear) {
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
   int v[kScanPer];
   int s = 0;
@@ -401,7 +403,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* __restri
   int run = block_exclusive(s) + offsets[blockIdx.x];
 #pragma unroll
   for (int q = 0; q < kScanPer; ++q) {
-    if (base + q < n) out[base + q] = run;
+    if (base + q < n) {
+      out[base + q] = run;
+      if (clear) in[base + q] = 0;
+    }
     run += v[q];
   }
 }
@@ -435,6 +440,62 @@ __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const 
     sp.item = item;
     sp.dense = 0;
     subs[s0 + k] = sp;
+  }
+}
+
+// k_sub_count, the scan of its counts and k_sub_fill in one block, for up to
+// kSubSingle bins: one launch in place of three, and the records are written
+// by all threads evenly instead of by each bin's thread.
+constexpr int kSubSingle = 16384;
+
+__global__ void __launch_bounds__(1024) k_subproblems(SortArgs s, const int* __restrict__ key_start, int P,
+                                                       int* __restrict__ bin_count, int* __restrict__ bin_start,
+                                                       int* __restrict__ sub_start, int* __restrict__ num_subs,
+                                                       SubProblem* __restrict__ subs) {
+  __shared__ int wsum[32];
+  const int nb = s.total_bins, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int chunk = (nb + 1023) / 1024;
+  const int lo = min(nb, (int)threadIdx.x * chunk), hi = min(nb, lo + chunk);
+  int mine = 0;
+  for (int b = lo; b < hi; ++b) {
+    const ItemDev& it = s.items[find_item<int>(s.bin_offsets, s.n_items, b)];
+    const int key = it.key_offset + (b - it.bin_offset) * it.geom.fine;
+    const int start = key_start[key], cnt = key_start[key + it.geom.fine] - start;
+    bin_count[b] = cnt;
+    bin_start[b] = start;
+    mine += (cnt + P - 1) / P;
+  }
+  int inc = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) wsum[w] = inc;
+  __syncthreads();
+  int before = 0, total = 0;
+  for (int k = 0; k < 32; ++k) {
+    before += k < w ? wsum[k] : 0;
+    total += wsum[k];
+  }
+  int run = before + inc - mine;
+  for (int b = lo; b < hi; ++b) {
+    sub_start[b] = run;
+    run += (bin_count[b] + P - 1) / P;
+  }
+  if (threadIdx.x == 0) *num_subs = total;
+  __syncthreads();
+  for (int t = threadIdx.x; t < total; t += 1024) {
+    const int b = find_item<int>(sub_start, nb, t);   // the last bin that starts at t or before: not an empty one
+    const int item = find_item<int>(s.bin_offsets, s.n_items, b);
+    const int off = (t - sub_start[b]) * P;
+    SubProblem sp;
+    sp.bin = b - s.bin_offsets[item];
+    sp.start = bin_start[b] + off;
+    sp.count = min(P, bin_count[b] - off);
+    sp.item = item;
+    sp.dense = 0;
+    subs[t] = sp;
   }
 }
 
@@ -589,16 +650,16 @@ constexpr int kScanSingle = 4 * kScanTile;
 
 int scan_launches(int n) { return n <= kScanSingle ? 1 : 3; }
 
-cudaError_t launch_scan(const int* in, int* out, int n, int* total, int* partials, cudaStream_t st) {
+cudaError_t launch_scan(int* in, int* out, int n, int* total, int* partials, bool clear, cudaStream_t st) {
   if (n <= kScanSingle) {
-    k_scan<<<1, 1024, 0, st>>>(in, out, n, total);
+    k_scan<<<1, 1024, 0, st>>>(in, out, n, total, clear);
     return cudaGetLastError();
   }
   const int tiles = (n + kScanTile - 1) / kScanTile;
   int* const offsets = partials + tiles;   // the scanned tile sums
   if (tiles > 0) k_scan_reduce<<<tiles, kScanThreads, 0, st>>>(in, n, partials);
-  k_scan<<<1, 1024, 0, st>>>(partials, offsets, tiles, total);
-  if (tiles > 0) k_scan_apply<<<tiles, kScanThreads, 0, st>>>(in, out, n, offsets);
+  k_scan<<<1, 1024, 0, st>>>(partials, offsets, tiles, total, false);
+  if (tiles > 0) k_scan_apply<<<tiles, kScanThreads, 0, st>>>(in, out, n, offsets, clear);
   return cudaGetLastError();
 }
 
@@ -627,14 +688,18 @@ cudaError_t launch_scatter(const SortArgs& s, const int* key_start, const int2* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_subproblem_count(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
-                                    int* sub_count, cudaStream_t st) {
-  k_sub_count<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_count);
-  return cudaGetLastError();
-}
+int subproblem_launches(int nbins) { return nbins <= kSubSingle ? 1 : 2 + scan_launches(nbins); }
 
-cudaError_t launch_subproblem_fill(const SortArgs& s, const int* bin_count, const int* bin_start, const int* sub_start,
-                                   int P, SubProblem* subs, cudaStream_t st) {
+cudaError_t launch_subproblems(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
+                               int* sub_count, int* sub_start, int* num_subs, int* partials, SubProblem* subs,
+                               cudaStream_t st) {
+  if (s.total_bins <= kSubSingle) {
+    k_subproblems<<<1, 1024, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_start, num_subs, subs);
+    return cudaGetLastError();
+  }
+  k_sub_count<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_count);
+  const cudaError_t e = launch_scan(sub_count, sub_start, s.total_bins, num_subs, partials, false, st);
+  if (e != cudaSuccess) return e;
   k_sub_fill<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, bin_count, bin_start, sub_start, P, subs);
   return cudaGetLastError();
 }
