@@ -159,6 +159,67 @@ __global__ void __launch_bounds__(32 * kScaleWarps)
   }
 }
 
+// The transform of a small 1-D FP64 item by direct sums, a warp per output,
+// lanes over the inputs: fhat(k) = 1 / c_k sum_l g_l e^(-2 pi i k l / n), and
+// g_l = sum_k fhat(k) / c_k e^(+2 pi i k l / n).  An SM does two FP64 lanes
+// per clock, so an FFT in one block (n = 512: 20 us) leaves the chip idle while
+// n N products over all SMs take about a microsecond; scaling and crop or
+// padding ride along.  Step of the exponent between a lane's terms: 32 k (or
+// 32 l) mod n, so its index moves by additions.
+__device__ __forceinline__ double2 warp_sum2(double2 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+  }
+  return v;
+}
+
+__global__ void __launch_bounds__(32 * kScaleWarps)
+    k_dft_crop(const ItemDev* __restrict__ items, const double2* __restrict__ roots, double2* __restrict__ out) {
+  const ItemDev& it = items[0];
+  const int N = it.N[0], n = it.geom.n[0], lane = threadIdx.x & 31;
+  const int a = blockIdx.x * kScaleWarps + (threadIdx.x >> 5);
+  if (a >= N) return;
+  const double2* g = static_cast<const double2*>(it.grid) + (int64_t)blockIdx.y * it.geom.grid_cells;
+  const int k = a < N / 2 ? a - N / 2 + n : a - N / 2;   // k mod n
+  int e = (int)((int64_t)k * lane % n);
+  const int step = (int)((int64_t)k * 32 % n);
+  double2 s = make_double2(0.0, 0.0);
+  for (int l = lane; l < n; l += 32) {
+    const double2 w = __ldg(roots + e), v = g[l];
+    s.x = fma(v.x, w.x, fma(v.y, w.y, s.x));
+    s.y = fma(v.y, w.x, fma(-v.x, w.y, s.y));
+    e += step;
+    e = e >= n ? e - n : e;
+  }
+  s = warp_sum2(s);
+  const double f = it.inv_c[0][a];
+  if (lane == 0) out[(int64_t)blockIdx.y * N + a] = make_double2(s.x * f, s.y * f);
+}
+
+__global__ void __launch_bounds__(32 * kScaleWarps)
+    k_pad_dft(const ItemDev* __restrict__ items, const double2* __restrict__ roots, const double2* __restrict__ in) {
+  const ItemDev& it = items[0];
+  const int N = it.N[0], n = it.geom.n[0], lane = threadIdx.x & 31;
+  const int l = blockIdx.x * kScaleWarps + (threadIdx.x >> 5);
+  if (l >= n) return;
+  const double2* h = in + (int64_t)blockIdx.y * N;
+  int e = (int)((int64_t)l * ((lane - N / 2 + (int64_t)n) % n) % n);   // lane < n: N <= n; both factors below n
+  const int step = (int)((int64_t)l * 32 % n);
+  double2 s = make_double2(0.0, 0.0);
+  for (int a = lane; a < N; a += 32) {
+    const double2 w = __ldg(roots + e), v = h[a];
+    const double f = it.inv_c[0][a], x = v.x * f, y = v.y * f;
+    s.x = fma(x, w.x, fma(-y, w.y, s.x));
+    s.y = fma(y, w.x, fma(x, w.y, s.y));
+    e += step;
+    e = e >= n ? e - n : e;
+  }
+  s = warp_sum2(s);
+  if (lane == 0) static_cast<double2*>(it.grid)[(int64_t)blockIdx.y * it.geom.grid_cells + l] = s;
+}
+
 }  // namespace
 
 int64_t scale_blocks(int64_t rows, int64_t row_length, bool batched) {
@@ -180,6 +241,19 @@ cudaError_t launch_pad_deconv(const ItemDev* items, const int* block_offsets, co
                               const void* in, int nrhs, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
   k_pad_deconv<Real><<<(unsigned)blocks, 32 * kScaleWarps, 0, st>>>(items, block_offsets, block_items, in, nrhs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dft_crop(const ItemDev* items, const double2* roots, int N, void* out, int nrhs, cudaStream_t st) {
+  k_dft_crop<<<dim3((N + kScaleWarps - 1) / kScaleWarps, nrhs), 32 * kScaleWarps, 0, st>>>(
+      items, roots, static_cast<double2*>(out));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pad_dft(const ItemDev* items, const double2* roots, int n, const void* in, int nrhs,
+                           cudaStream_t st) {
+  k_pad_dft<<<dim3((n + kScaleWarps - 1) / kScaleWarps, nrhs), 32 * kScaleWarps, 0, st>>>(
+      items, roots, static_cast<const double2*>(in));
   return cudaGetLastError();
 }
 

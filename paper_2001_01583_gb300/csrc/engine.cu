@@ -15,6 +15,11 @@ constexpr size_t kSmemBudget = 200 * 1024;   // per block (the opt-in limit is 2
 constexpr int kPencilBlocksPerSm = 16;       // pencil subproblems per SM a point set is cut into at least
 constexpr size_t kSmemTarget = 100 * 1024;   // thread-per-point tiles: aim at two blocks per SM
 
+// 1-D FP64 transforms of one item small enough for the direct sum over the
+// chip (k_dft_crop, k_pad_dft): 2^20 complex products take 7 us at the chip's
+// FP64 rate, an FFT in one block 20 us from n = 512 on.
+constexpr int64_t kDirectProducts = (int64_t)1 << 20;
+
 #define CK(call)                                                             \
   do {                                                                       \
     cudaError_t e_ = (call);                                                 \
@@ -293,6 +298,7 @@ Engine::~Engine() {
   for (auto& fc : fclasses) {
     destroy_fft_plans(fc);
     free_dev(fc.buf);
+    free_dev(fc.roots);
   }
   for (double* t : tables) cudaFree(t);
   free_dev(err_flag);
@@ -396,6 +402,15 @@ int Engine::build_fft() {
     TRY(alloc_dev(fc.buf, (size_t)fc.grids * (size_t)fc.cells * csize, device_bytes));
     cufftHandle h;
     TRY(fft_handle(fc, single ? 1 : fc.grids, &h));
+    if (single && fc.d == 1 && precision == NFFT_FP64 && fc.n[0] * specs[0].N[0] <= kDirectProducts) {
+      std::vector<double> t(2 * (size_t)fc.n[0]);   // e^(2 pi i j / n)
+      for (int64_t j = 0; j < fc.n[0]; ++j) {
+        t[2 * j] = std::cos(2.0 * M_PI * j / fc.n[0]);
+        t[2 * j + 1] = std::sin(2.0 * M_PI * j / fc.n[0]);
+      }
+      TRY(alloc_dev(fc.roots, sizeof(double) * t.size(), device_bytes));
+      CK(cudaMemcpy(fc.roots, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice));
+    }
   }
   return NFFT_OK;
 }
@@ -941,6 +956,10 @@ int Engine::run_fft(FClass& fc, int batch, int64_t grid_offset, int direction) {
   return r == CUFFT_SUCCESS ? NFFT_OK : NFFT_ERR_CUFFT;
 }
 
+bool Engine::direct_dft(const FClass& fc, int nr) const {
+  return single && fc.d == 1 && precision == NFFT_FP64 && fc.n[0] * items[0].N[0] * nr <= kDirectProducts;
+}
+
 // ===========================================================================
 // profiling
 
@@ -1374,10 +1393,16 @@ int Engine::adjoint_single(const void* f, void* fhat, int R) {
     }
     TRY(stage_end(&ev));
     TRY(stage_begin(NFFT_STAGE_FFT, &ev));
+    void* out = static_cast<char*>(fhat) + (int64_t)r0 * it.NN * (int64_t)csize;
+    if (direct_dft(fc, nr)) {
+      CK(launch_dft_crop(d_items, fc.roots, it.N[0], out, nr, stream));
+      ++kernel_launches;
+      TRY(stage_end(&ev));
+      continue;
+    }
     TRY(run_fft(fc, nr, item_grid_offset[0], CUFFT_FORWARD));
     TRY(stage_end(&ev));
     TRY(stage_begin(NFFT_STAGE_DECONV, &ev));
-    void* out = static_cast<char*>(fhat) + (int64_t)r0 * it.NN * (int64_t)csize;
     const int64_t cblocks = scale_blocks(it.NN / it.N[it.geom.d - 1] * nr, it.N[it.geom.d - 1], false);
     CK(precision == NFFT_FP64 ? launch_deconv_crop<double>(d_items, nullptr, nullptr, cblocks, out, nr, stream)
                               : launch_deconv_crop<float>(d_items, nullptr, nullptr, cblocks, out, nr, stream));
@@ -1393,16 +1418,23 @@ int Engine::forward_single(const void* fhat, void* f, int R) {
   for (int r0 = 0; r0 < R; r0 += rhs_cap) {
     const int nr = (R - r0) < rhs_cap ? (R - r0) : rhs_cap;
     EventPair ev{};
-    TRY(stage_begin(NFFT_STAGE_PAD, &ev));
     const void* hin = static_cast<const char*>(fhat) + (int64_t)r0 * it.NN * (int64_t)csize;
-    const int64_t pblocks = scale_blocks(fc.cells / fc.n[fc.d - 1] * nr, fc.n[fc.d - 1], false);
-    CK(precision == NFFT_FP64 ? launch_pad_deconv<double>(d_items, nullptr, nullptr, pblocks, hin, nr, stream)
-                              : launch_pad_deconv<float>(d_items, nullptr, nullptr, pblocks, hin, nr, stream));
-    kernel_launches += pblocks > 0 ? 1 : 0;
-    TRY(stage_end(&ev));
-    TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
-    TRY(run_fft(fc, nr, item_grid_offset[0], CUFFT_INVERSE));
-    TRY(stage_end(&ev));
+    if (direct_dft(fc, nr)) {
+      TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
+      CK(launch_pad_dft(d_items, fc.roots, (int)fc.n[0], hin, nr, stream));
+      ++kernel_launches;
+      TRY(stage_end(&ev));
+    } else {
+      TRY(stage_begin(NFFT_STAGE_PAD, &ev));
+      const int64_t pblocks = scale_blocks(fc.cells / fc.n[fc.d - 1] * nr, fc.n[fc.d - 1], false);
+      CK(precision == NFFT_FP64 ? launch_pad_deconv<double>(d_items, nullptr, nullptr, pblocks, hin, nr, stream)
+                                : launch_pad_deconv<float>(d_items, nullptr, nullptr, pblocks, hin, nr, stream));
+      kernel_launches += pblocks > 0 ? 1 : 0;
+      TRY(stage_end(&ev));
+      TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
+      TRY(run_fft(fc, nr, item_grid_offset[0], CUFFT_INVERSE));
+      TRY(stage_end(&ev));
+    }
     TRY(stage_begin(NFFT_STAGE_INTERP, &ev));
     if (it.M > 0) {
       void* fout = static_cast<char*>(f) + (int64_t)r0 * it.M * (int64_t)csize;
@@ -1719,6 +1751,8 @@ int Engine::set_option(int option, int64_t value) {
         destroy_fft_plans(fc);
         device_bytes -= (int64_t)fc.grids * fc.cells * (int64_t)csize;
         free_dev(fc.buf);
+        if (fc.roots) device_bytes -= (int64_t)sizeof(double2) * fc.n[0];
+        free_dev(fc.roots);
       }
       fclasses.clear();
       rhs_cap = (int)value;

@@ -53,6 +53,7 @@ struct FClass {
   int64_t cells;
   int grids;                  // grids in the buffer
   void* buf = nullptr;
+  double2* roots = nullptr;     // e^(2 pi i j / n), j < n (1-D FP64 transforms by direct sums)
   std::map<int, cufftHandle> plans;
   bool owner_written = false;   // every grid of the class is written whole by the owner kernel
   // pruned 3-D FFT (one item): 1-D along dimension 0 over the grid, 2-D over
@@ -134,6 +135,7 @@ class Engine {
   template <typename Real> int ewald_forces_impl(const void* q, double L, double alpha, double* F);
   int run_fft(FClass& fc, int batch, int64_t grid_offset, int direction);
   bool fft_pruned(const FClass& fc) const;
+  bool direct_dft(const FClass& fc, int nr) const;
   int build_pruned(FClass& fc);
   void destroy_fft_plans(FClass& fc);
   int fft_handle(FClass& fc, int batch, cufftHandle* out);

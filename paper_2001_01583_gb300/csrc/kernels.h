@@ -191,4 +191,10 @@ template <typename Real>
 cudaError_t launch_pad_deconv(const ItemDev* items, const int* block_offsets, const int* block_items, int64_t blocks,
                               const void* in, int nrhs, cudaStream_t st);
 
+// Small 1-D FP64 items (items[0]): the DFT by direct sums, with the scaling
+// and the crop or padding.  roots: e^(2 pi i j / n); N, n: the rows to write.
+cudaError_t launch_dft_crop(const ItemDev* items, const double2* roots, int N, void* out, int nrhs, cudaStream_t st);
+cudaError_t launch_pad_dft(const ItemDev* items, const double2* roots, int n, const void* in, int nrhs,
+                           cudaStream_t st);
+
 }  // namespace gbnfft
