@@ -506,9 +506,11 @@ __global__ void __launch_bounds__(1024) k_subproblems(SortArgs s, const int* __r
 // shared-memory broadcasts (SubProblem::dense).  The scatter writes 4 bytes per point to a random place
 // instead of 20 in five arrays (32-byte sectors: 5 of them; M = 3 10^7: 1.23
 // -> 0.21 ms); the coordinates are gathered here instead, and the records go
-// out in order (1.04 ms with the sort, M = 10^6 uniform without it: 19 us).  Bitonic sort of
-// 32-bit keys (cell, slot): a step of distance 32 or less stays inside a
-// warp's 64 keys, so only the longer ones need a block barrier.
+// out in order (0.81 ms with the sort, M = 10^6 uniform without it: 21 us).  Bitonic sort of
+// 32-bit keys (cell, slot), four per thread in registers: a step's partner is
+// in the thread, in another lane (a shuffle) or, from distance 128 on, in
+// another warp (shared memory, 6 of the 55 steps; all steps in shared memory:
+// 1.04 ms).
 constexpr int kRefine = 1024;
 constexpr int kRefineThreads = 256;
 constexpr int kRefinePer = kRefine / kRefineThreads;
@@ -517,7 +519,9 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
                                                            const int* __restrict__ num_subs, int* __restrict__ perm,
                                                            uint32_t* __restrict__ local, float* __restrict__ d0,
                                                            float* __restrict__ d1, float* __restrict__ d2) {
-  __shared__ uint32_t key[kRefine], loc[kRefine];
+  static_assert(kRefinePer == 4, "four elements per thread");
+  __shared__ __align__(16) uint32_t key[kRefine];
+  __shared__ uint32_t loc[kRefine];
   __shared__ int idx[kRefine];
   __shared__ float del[3][kRefine];
   if ((int)blockIdx.x >= *num_subs) return;
@@ -566,8 +570,6 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
         idx[i] = j[q];
         loc[i] = packed;
         key[i] = k << 10 | (uint32_t)i;
-      } else if (i < size) {
-        key[i] = 0xffffffffu;
       }
     }
     __syncthreads();
@@ -587,21 +589,46 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
       __syncthreads();
       continue;
     }
+    // element 4 t + r of the sort in register r of thread t
+    const int first_e = kRefinePer * threadIdx.x;
+    uint32_t e[kRefinePer];
+#pragma unroll
+    for (int r = 0; r < kRefinePer; ++r) e[r] = first_e + r < cnt ? key[first_e + r] : 0xffffffffu;
     for (int k = 2; k <= size; k *= 2) {
-      for (int d = k / 2; d > 0; d /= 2) {
-        for (int t = threadIdx.x; t < size / 2; t += kRefineThreads) {
-          const int a = 2 * t - (t & (d - 1));
-          const uint32_t u = key[a], v = key[a + d];
-          if ((u > v) == ((a & k) == 0)) {
-            key[a] = v;
-            key[a + d] = u;
-          }
-        }
-        // the next step is (k, d / 2) or (2 k, k)
-        if (d > 32 || (d == 1 && k > 32)) __syncthreads();
-        else __syncwarp();
+      for (int d = k / 2; d >= 4 * 32; d /= 2) {   // partner in another warp
+        __syncthreads();
+        *reinterpret_cast<uint4*>(key + first_e) = make_uint4(e[0], e[1], e[2], e[3]);
+        __syncthreads();
+        const uint4 o = *reinterpret_cast<const uint4*>(key + (first_e ^ d));
+        const bool low = ((first_e & d) == 0) == ((first_e & k) == 0);
+        e[0] = low ? min(e[0], o.x) : max(e[0], o.x);
+        e[1] = low ? min(e[1], o.y) : max(e[1], o.y);
+        e[2] = low ? min(e[2], o.z) : max(e[2], o.z);
+        e[3] = low ? min(e[3], o.w) : max(e[3], o.w);
       }
+      for (int d = min(k / 2, 64); d >= 4; d /= 2) {   // in another lane
+        const bool low = ((first_e & d) == 0) == ((first_e & k) == 0);
+#pragma unroll
+        for (int r = 0; r < kRefinePer; ++r) {
+          const uint32_t o = __shfl_xor_sync(0xffffffffu, e[r], d / 4);
+          e[r] = low ? min(e[r], o) : max(e[r], o);
+        }
+      }
+      const bool up = (first_e & k) == 0;   // in this thread: (0, 2), (1, 3), then (0, 1), (2, 3)
+      auto swap = [](uint32_t& x, uint32_t& y, bool ascending) {
+        const uint32_t lo = min(x, y), hi = max(x, y);
+        x = ascending ? lo : hi;
+        y = ascending ? hi : lo;
+      };
+      if (k >= 4) {
+        swap(e[0], e[2], up);
+        swap(e[1], e[3], up);
+      }
+      swap(e[0], e[1], k == 2 ? true : up);
+      swap(e[2], e[3], k == 2 ? false : up);
     }
+    __syncthreads();
+    *reinterpret_cast<uint4*>(key + first_e) = make_uint4(e[0], e[1], e[2], e[3]);
     __syncthreads();
     int cells = 0;   // of this thread's points, those that begin a cell
     for (int i = threadIdx.x; i < cnt; i += kRefineThreads) {
