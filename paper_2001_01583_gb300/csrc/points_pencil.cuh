@@ -32,11 +32,12 @@
 //
 // Measured on GB300 (Kaiser-Bessel, sigma = 2, spread / interpolation, against
 // the kernels of points_planes.cuh and points_gm.cuh at their default bins):
-//   N = 64^3, M = 10^6, m = 4, uniform: 229 / 214 us from 441 / 248
-//     clustered (32 clusters, std 0.02): 218 / 179 us from 566 / 288
-//   N = 256^3, M = 3 10^7, m = 3, 64 clusters, std 0.01: 3.6 / 2.1 ms from
+//   N = 64^3, M = 10^6, m = 4, uniform: 222 / 206 us from 441 / 248
+//     clustered (32 clusters, std 0.02): 209 / 180 us from 566 / 288
+//   N = 90 x 128 x 74, M = 777777, m = 5: 311 / 532 us from 1069 / 989
+//   N = 256^3, M = 3 10^7, m = 3, 64 clusters, std 0.01: 3.5 / 2.0 ms from
 //     14.9 / 5.0
-//   N = 128^3, 393216 ions, m = 6: 384 us from 2471 (spread only)
+//   N = 128^3, 393216 ions, m = 6: 388 us from 2471 (spread only)
 #pragma once
 
 #include "points_planes.cuh"
@@ -46,13 +47,18 @@ namespace gbnfft {
 // The pencil kernels' shape for W taps and NR x NR squares.
 template <int W, int NR>
 struct PencilShape {
-  static constexpr int THREADS = 32 * NR * NR;
-  static constexpr int PARTS = NR == 2 ? 2 : 3;        // threads that stage one point
-  static constexpr int BP = NR == 2 ? 64 : (NR == 3 ? 96 : 160);   // points per batch (a multiple of 32)
+  // columns per lane: a warp's part of the tile is 4 C rows by 8 columns
+  // (C = 4 reads fewer weights per point and meets more idle lanes: 243 us
+  // against 229 for N = 64^3, M = 10^6, 8 taps, and 3.9 against 3.6 ms for 6
+  // taps on the largest configuration)
+  static constexpr int C = 2;
+  static constexpr int ROWS = 4 * C, WARPS = 8 * NR / ROWS * NR, THREADS = 32 * WARPS;
+  // threads that stage one point, and points per batch (a multiple of 32)
+  static constexpr int PARTS = NR == 2 ? 2 : 3, BP = NR == 2 ? THREADS / 2 : 96;
   // resident blocks asked of the compiler
-  static constexpr int MIN_BLOCKS = NR == 2 ? (W <= 6 ? 6 : 5) : (W <= 12 ? 2 : 1);
-  static constexpr int PAD = 8;                        // zeros on each side of wy and wx
-  static constexpr int LEN = (W + 2 * PAD + 3) / 4 * 4;
+  static constexpr int MIN_BLOCKS = NR == 2 ? (W <= 6 ? 7 : 5) : (W <= 12 ? 2 : 1);
+  static constexpr int PADX = 8, PADY = ROWS;   // zeros on each side of wx and wy
+  static constexpr int LENX = (W + 2 * PADX + 3) / 4 * 4, LENY = (W + 2 * PADY + 3) / 4 * 4;
   static_assert(PARTS * BP <= THREADS, "a thread stages at most one part");
 };
 
@@ -62,8 +68,8 @@ template <int W, int NR>
 struct PencilRow {
   using S = PencilShape<W, NR>;
   static constexpr int WY = (W + 3) / 4 * 4;
-  static constexpr int WX = WY + S::LEN;
-  static constexpr int S4 = (WX + 2 * S::LEN + 3) / 4;
+  static constexpr int WX = WY + S::LENY;
+  static constexpr int S4 = (WX + 2 * S::LENX + 3) / 4;
   static constexpr int STRIDE = 4 * (S4 % 2 ? S4 : S4 + 1);
   static constexpr size_t BYTES = (size_t)(S::BP + 1) * STRIDE * sizeof(float);   // a row of zeros after the points'
 };
@@ -72,7 +78,7 @@ struct PencilRow {
 template <int W, int NR>
 constexpr size_t pencil_smem_bytes() {
   using S = PencilShape<W, NR>;
-  return PencilRow<W, NR>::BYTES + (size_t)NR * NR * S::BP * 16 + (size_t)S::BP * sizeof(uint32_t);
+  return PencilRow<W, NR>::BYTES + (size_t)S::WARPS * S::BP * 16 + (size_t)S::BP * sizeof(uint32_t);
 }
 
 __device__ __forceinline__ void sts_f4(uint32_t a, float x, float y, float z, float w) {
@@ -146,7 +152,7 @@ struct PencilFetch {
     }
     if (part() == S::PARTS - 2) {
       window_taps<W>(win, 1, db, w);
-      sts_row<W>(row + 4u * (R::WY + S::PAD), w);
+      sts_row<W>(row + 4u * (R::WY + S::PADY), w);
     }
     if (part() == S::PARTS - 1) {
       rec[t] = loc;
@@ -154,7 +160,7 @@ struct PencilFetch {
 #pragma unroll
       for (int i = 0; i < W; i += 2) {
         const float2 p = cscale(v, w[i]), q = cscale(v, w[i + 1]);
-        sts_f4(row + 4u * (R::WX + 2 * (S::PAD + i)), p.x, p.y, q.x, q.y);
+        sts_f4(row + 4u * (R::WX + 2 * (S::PADX + i)), p.x, p.y, q.x, q.y);
       }
     }
   }
@@ -194,12 +200,12 @@ __device__ __forceinline__ int pencil_list(const uint32_t* rec, uint32_t wt_a, u
     const uint32_t loc = rec[t];   // t < BP; stale past nb
     const int dy = y0 - unpack_local(loc, 3, 1), dx = x0 - unpack_local(loc, 3, 2);
     const int l0 = unpack_local(loc, 3, 0);
-    const bool reach = t < nb && dy > -S::PAD && dy < W && dx > -S::PAD && dx < W;
+    const bool reach = t < nb && dy > -S::PADY && dy < W && dx > -S::PADX && dx < W;
     const unsigned mask = __ballot_sync(0xffffffffu, reach);
     if (reach) {
       const uint32_t row = wt_a + 4u * (uint32_t)(t * R::STRIDE);
       sts_u4(list_a + 16u * (uint32_t)(n + __popc(mask & ((1u << lane) - 1u))), row,
-             row + 4u * (uint32_t)(R::WY + S::PAD + dy), row + 4u * R::WX + 8u * (uint32_t)(S::PAD + dx), (uint32_t)l0);
+             row + 4u * (uint32_t)(R::WY + S::PADY + dy), row + 4u * R::WX + 8u * (uint32_t)(S::PADX + dx), (uint32_t)l0);
     }
     if (mask) last = __shfl_sync(0xffffffffu, l0, 31 - __clz(mask));
     n += __popc(mask);
@@ -223,10 +229,11 @@ __device__ __forceinline__ bool pencil_sub(const PointKernelArgs<float>& a, SubP
   return true;
 }
 
-// The pencil's first tile column and plane in the grid, and this lane's two
-// columns (flat index inside a plane).
+// The pencil's first plane in the grid, and this lane's columns (flat index
+// inside a plane).
+template <int C>
 struct PencilCols {
-  int z0, col[2];
+  int z0, col[C];
   __device__ __forceinline__ PencilCols(const ItemDev& it, int bin, int y0, int x0, int lane) {
     const GridGeom& g = it.geom;
     int bc[kMaxDim];
@@ -235,23 +242,25 @@ struct PencilCols {
     z0 = bc[0] * g.bin[0] + s;
     const int x = wrap_mod(bc[2] * g.bin[2] + s + x0 + (lane & 7), g.n[2]);
 #pragma unroll
-    for (int c = 0; c < 2; ++c)
+    for (int c = 0; c < C; ++c)
       col[c] = wrap_mod(bc[1] * g.bin[1] + s + y0 + (lane >> 3) + 4 * c, g.n[1]) * g.n[2] + x;
   }
 };
 
 template <int W, int NR>
-__global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR>::MIN_BLOCKS) k_spread_pencil(PointKernelArgs<float> a) {
+__global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR>::MIN_BLOCKS)
+    k_spread_pencil(PointKernelArgs<float> a) {
   using S = PencilShape<W, NR>;
   using R = PencilRow<W, NR>;
+  constexpr int C = S::C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* wt = reinterpret_cast<float*>(smem_raw);
-  uint4* list = reinterpret_cast<uint4*>(smem_raw + R::BYTES);   // [squares][BP]
-  uint32_t* rec = reinterpret_cast<uint32_t*>(list + NR * NR * S::BP);
+  uint4* list = reinterpret_cast<uint4*>(smem_raw + R::BYTES);   // [warps][BP]
+  uint32_t* rec = reinterpret_cast<uint32_t*>(list + S::WARPS * S::BP);
   SubProblem sub;
   if (!pencil_sub(a, sub)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y0 = warp / NR * 8, x0 = warp % NR * 8;
+  const int y0 = warp / NR * S::ROWS, x0 = warp % NR * 8;
   for (int e = threadIdx.x; e < (S::BP + 1) * R::STRIDE / 4; e += S::THREADS)
     reinterpret_cast<float4*>(wt)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   const ItemDev& it = a.items[sub.item];
@@ -260,29 +269,30 @@ __global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR
   const int r = blockIdx.y;
   const float2* f_in = static_cast<const float2*>(call.in) + (int64_t)r * it.M;
   float2* grid = static_cast<float2*>(it.grid) + (int64_t)r * g.grid_cells;
-  const PencilCols pc(it, sub.bin, y0, x0, lane);
+  const PencilCols<C> pc(it, sub.bin, y0, x0, lane);
   const int n0 = g.n[0], plane = g.n[1] * g.n[2];
-  float2* const g0 = grid + pc.col[0];
-  float2* const g1 = grid + pc.col[1];
   const uint32_t wt_a = (uint32_t)__cvta_generic_to_shared(wt);
   const uint32_t wy_l = 4u * (uint32_t)(lane >> 3), wx_l = 8u * (uint32_t)(lane & 7);
   const uint32_t list_a = (uint32_t)__cvta_generic_to_shared(list + warp * S::BP);
   // the window: real and imaginary parts of W cells per column, pairs along
   // dimension 0 (a paired FMA takes two neighbouring weights as they lie)
-  Pair re[2][W / 2], im[2][W / 2];
+  Pair re[C][W / 2], im[C][W / 2];
 #pragma unroll
-  for (int i = 0; i < W / 2; ++i) re[0][i] = re[1][i] = im[0][i] = im[1][i] = 0;
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int i = 0; i < W / 2; ++i) re[c][i] = im[c][i] = 0;
   int cur = -1;        // plane of the window's first cell (in the pencil)
   bool live = false;   // the window holds something
   // the window's first plane to the grid, the window one plane on
   auto flush = [&]() {
-    const int64_t zo = (int64_t)wrap_mod(pc.z0 + cur, n0) * plane;
-    const float2 v0 = make_float2(halves(re[0][0]).x, halves(im[0][0]).x);
-    const float2 v1 = make_float2(halves(re[1][0]).x, halves(im[1][0]).x);
-    if (v0.x != 0.f || v0.y != 0.f) grid_add(g0 + zo, v0);
-    if (v1.x != 0.f || v1.y != 0.f) grid_add(g1 + zo, v1);
+    float2* const zp = grid + (int64_t)wrap_mod(pc.z0 + cur, n0) * plane;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < C; ++c) {
+      const float2 v = make_float2(halves(re[c][0]).x, halves(im[c][0]).x);
+      if (v.x != 0.f || v.y != 0.f) grid_add(zp + pc.col[c], v);
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
       window_step<W>(re[c], 0.f);
       window_step<W>(im[c], 0.f);
     }
@@ -296,18 +306,24 @@ __global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR
   };
   auto add = [&](const uint4& e) {
     Pair wz[W / 2];
-    const float ya0 = lds_f1(e.y + wy_l), ya1 = lds_f1(e.y + wy_l + 16u);
+    float wy[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) wy[c] = lds_f1(e.y + wy_l + 16u * (uint32_t)c);
     const float2 v = lds_f2(e.z + wx_l);
     lds_pairs<W>(e.x, wz);
-    const Pair r0 = pair(v.x * ya0, v.x * ya0), i0 = pair(v.y * ya0, v.y * ya0);
-    const Pair r1 = pair(v.x * ya1, v.x * ya1), i1 = pair(v.y * ya1, v.y * ya1);
+    Pair pr[C], pi[C];
 #pragma unroll
-    for (int i = 0; i < W / 2; ++i) {
-      re[0][i] = pair_fma(wz[i], r0, re[0][i]);
-      im[0][i] = pair_fma(wz[i], i0, im[0][i]);
-      re[1][i] = pair_fma(wz[i], r1, re[1][i]);
-      im[1][i] = pair_fma(wz[i], i1, im[1][i]);
+    for (int c = 0; c < C; ++c) {
+      pr[c] = pair(v.x * wy[c], v.x * wy[c]);
+      pi[c] = pair(v.y * wy[c], v.y * wy[c]);
     }
+#pragma unroll
+    for (int i = 0; i < W / 2; ++i)
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        re[c][i] = pair_fma(wz[i], pr[c], re[c][i]);
+        im[c][i] = pair_fma(wz[i], pi[c], im[c][i]);
+      }
   };
   PencilFetch<W, NR> fetch;
   const int end = sub.start + sub.count;
@@ -323,7 +339,11 @@ __global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR
       const uint32_t la = list_a + 16u * (uint32_t)k;
       if (lds_i1(la + 12u) == cur && lds_i1(la + 60u) == cur) {   // planes ascend: all four are the window's
 #pragma unroll
-        for (int q = 0; q < 4; ++q) add(lds_u4(la + 16u * (uint32_t)q));
+        for (int q = 0; q < 4; q += 2) {   // two entries on their way before the first is used
+          const uint4 e0 = lds_u4(la + 16u * (uint32_t)q), e1 = lds_u4(la + 16u * (uint32_t)q + 16u);
+          add(e0);
+          add(e1);
+        }
       } else {
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
@@ -351,7 +371,7 @@ __global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR
 //     so for the others.
 template <int W, int NR>
 struct SlabShape {
-  static constexpr int THREADS = NR == 2 || W >= 14 ? 128 : 256;
+  static constexpr int THREADS = W <= 6 ? 192 : NR == 2 || W >= 14 ? 128 : 256;
   static constexpr int SIDE = 8 * NR;   // tile columns per dimension
   // pitch of a tile row in cells, and whether a lane's rows are neighbours
   // (row q PASSES + k) or Q apart (q + Q k): the fewest wavefronts over all
@@ -359,7 +379,10 @@ struct SlabShape {
   static constexpr int PITCH = W == 2 ? 18 : W == 4 ? 20 : W == 6 ? 22 : W == 8 ? 20 : W <= 12 ? 26 : W == 14 ? 30 : 24;
   static constexpr bool NEIGHBOURS = W == 8 || W == 12;
   static constexpr int PLANE = SIDE * PITCH;
-  static constexpr int AHEAD = NR == 2 ? 7 : W == 10 ? 4 : W == 12 ? 2 : 1;   // planes of points a slab serves
+  // (8 taps, uniform, M = 10^6: 254 us for 3 planes, 236 for 4, 213 for 7, 206
+  // for 9, 210 for 12; 96000 points, three right-hand sides: 346, 259, 219,
+  // 195, 180.  More planes mean fewer reloads and fewer resident blocks)
+  static constexpr int AHEAD = W == 8 ? 9 : NR == 2 ? 7 : W == 12 ? 2 : 1;   // planes of points a slab serves
   static constexpr int PLANES = AHEAD + W - 1;
   static constexpr int Q = 32 / W, PASSES = (W + Q - 1) / Q;
   static constexpr bool FULL = 32 % W == 0 && Q * PASSES == W;
@@ -546,6 +569,8 @@ __global__ void __launch_bounds__(SlabShape<W, NR>::THREADS) k_interp_pencil(Poi
   }
 }
 
-#define GBNFFT_PENCIL_CASES(X) X(2, 2) X(4, 2) X(6, 2) X(8, 2) X(10, 3) X(12, 3) X(14, 3) X(16, 3)
+// Taps and squares per side: tiles of 16 x 16 columns to 10 taps (10 taps on 24
+// x 24: 412 / 645 us in place of 311 / 532 above), 24 x 24 beyond.
+#define GBNFFT_PENCIL_CASES(X) X(2, 2) X(4, 2) X(6, 2) X(8, 2) X(10, 2) X(12, 3) X(14, 3) X(16, 3)
 
 }  // namespace gbnfft
