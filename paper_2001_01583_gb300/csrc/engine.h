@@ -92,7 +92,7 @@ class Engine {
   int set_points_single(const double* x);
   int set_points_batch(const double* const* x);
   int adjoint_single(const void* f, void* fhat, int R);
-  int forward_single(const void* fhat, void* f, int R);
+  int forward_single(const void* fhat, void* f, int R, int cap = 0);   // cap: grids to use at once (at least rhs_cap)
   int adjoint_batch(const void* const* f, void* const* fhat);
   int forward_batch(const void* const* fhat, void* const* f);
   int sync();
@@ -138,6 +138,7 @@ class Engine {
   bool direct_dft(const FClass& fc, int nr) const;
   int build_pruned(FClass& fc);
   void destroy_fft_plans(FClass& fc);
+  int force_grids();
   int fft_handle(FClass& fc, int batch, cufftHandle* out);
   int blocks_per_sm(const void* fn, int threads, size_t smem);
   int stage_begin(int stage, EventPair* ev);
