@@ -164,8 +164,19 @@ __device__ __forceinline__ double window_psi<double>(const WindowDev& w, int t, 
 // are E + x O and E - x O.  Two FP32 taps cost 5 paired FMAs and 2 FMAs; the
 // formula (window_psi) costs 4 special-function instructions and about 16
 // others per tap, in FP64 about 110 FP64 operations against 11.  x is exact
-// to 2^-24 where u = delta + m - s would round at the size of m.  A window cut
-// at |u| = m is 0 there: its last tap at delta = 0.
+// to 2^-24 where u = delta + m - s would round at the size of m.
+
+// A window cut at |u| = m is 0 from there on: its outer taps where u, rounded
+// as window_psi rounds it, reaches the cut (delta = 0, or within rounding of a
+// cell's ends).
+template <int W, typename Real>
+__device__ __forceinline__ void cut_taps(const WindowDev& win, Real delta, Real* w) {
+  if (win.kind == 0) return;
+  const Real base = delta + (Real)(win.m - win.shift), last = base - (Real)(W - 1), m2 = (Real)win.m * (Real)win.m;
+  if (!(base * base < m2)) w[0] = (Real)0;
+  if (!(last * last < m2)) w[W - 1] = (Real)0;
+}
+
 template <int W>
 __device__ __forceinline__ void window_taps(const WindowDev& win, int t, float delta, float* w) {
   const float4* c = reinterpret_cast<const float4*>(win.polyf[t]);
@@ -184,7 +195,7 @@ __device__ __forceinline__ void window_taps(const WindowDev& win, int t, float d
     w[i] = fmaf(x, p.y, p.x);
     w[W - 1 - i] = fmaf(-x, p.y, p.x);
   }
-  if (win.kind != 0 && delta == 0.0f) w[W - 1] = 0.0f;
+  cut_taps<W>(win, delta, w);
 }
 template <int W>
 __device__ __forceinline__ void window_taps(const WindowDev& win, int t, double delta, double* w) {
@@ -199,7 +210,7 @@ __device__ __forceinline__ void window_taps(const WindowDev& win, int t, double 
     w[i] = fma(x, p.y, p.x);
     w[W - 1 - i] = fma(-x, p.y, p.x);
   }
-  if (win.kind != 0 && delta == 0.0) w[W - 1] = 0.0;
+  cut_taps<W>(win, delta, w);
 }
 
 // One of them, tap k (kernels whose lanes take different taps).
@@ -211,7 +222,10 @@ __device__ __forceinline__ double window_tap(const WindowDev& win, int t, double
   double2 p = __ldg(c + kPolyD - 1);
 #pragma unroll
   for (int q = kPolyD - 2; q >= 0; --q) p = cmad(p, s, __ldg(c + q));
-  if (win.kind != 0 && delta == 0.0 && k == taps - 1) return 0.0;
+  if (win.kind != 0) {
+    const double u = delta + (double)(win.m - win.shift) - (double)k, m = (double)win.m;
+    if (!(u * u < m * m)) return 0.0;
+  }
   return fma(mirror ? -x : x, p.y, p.x);
 }
 

@@ -41,3 +41,28 @@ def test_polynomial_windows(window, m, precision, sparse):
     for got, ref in ((a, S.adjoint(x, f, N, 2.0, m, WIN[window])), (b, S.forward(x, fh, N, 2.0, m, WIN[window]))):
         err = np.max(np.abs(got.cpu().numpy() - ref)) / np.sqrt(np.mean(np.abs(ref) ** 2))
         assert err <= tol, (window, m, err)
+
+
+@pytest.mark.parametrize("window", list(WIN))
+def test_offsets_within_rounding_of_a_node(window):
+    """A narrow FP32 window is cut where the formula's rounded argument reaches the cut: the kernels that take the
+    polynomials (a tile) against the one that takes the formula (a warp per point), 1e-5 of the rms; a tap that one of
+    them keeps would be 1e-3."""
+    from paper_2001_01583_gb300 import Plan, _lib
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    N, M = (64,), 60
+    x = ((np.arange(M) - 30) / 128.0 + np.repeat([2.0 ** -34, -2.0 ** -34, 2.0 ** -40], 20))[:, None]
+    f, fh = inputs.complex_normal(M, seed=73), inputs.complex_normal(N, seed=74)
+    out = []
+    for sparse in (-1, 1 << 20):
+        with Plan(N, M, 2.0, 2, window, "fp32") as p:
+            p.set_option(_lib.OPT_SPARSE_POINTS, sparse)
+            p.set_option(_lib.OPT_SPARSE_POINTS_INTERP, sparse)
+            p.set_points(torch.from_numpy(x).cuda())
+            a = p.adjoint(torch.from_numpy(f).to(torch.complex64).cuda())
+            b = p.forward(torch.from_numpy(fh).to(torch.complex64).cuda())
+            p.sync()
+            out.append((a.cpu().numpy(), b.cpu().numpy()))
+    for got, ref in zip(*out):
+        assert np.max(np.abs(got - ref)) <= 1e-5 * np.sqrt(np.mean(np.abs(ref) ** 2)), window
