@@ -253,7 +253,7 @@ struct GridGeom {
   int tile[kMaxDim];         // bin + W - 1 (unused dims = 1)
   int64_t grid_cells;        // prod n
   int tile_cells;            // prod tile
-  int fine;                  // sort keys per bin: 1, or bin[0] (a bin's points in the order of their plane)
+  int fine;                  // sort keys per bin: 1, or its planes (a pencil's points in their order)
 };
 
 // One transform of a batch (a single plan is a batch of one), as the

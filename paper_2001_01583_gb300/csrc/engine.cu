@@ -593,9 +593,11 @@ int Engine::build_layout() {
                !owner_enabled && !c.tensor && !c.tensor_interp && pl.fn &&
                (double)s.M * pl.edge * pl.edge >= (double)n[0] * (double)n[1] * (double)n[2];
     if (c.pencil) {
+      // the same bins for every grid size, so that the items of a batch share
+      // their launches
       const int want[3] = {(1 << local_bits(3)) - 1, pl.edge, pl.edge};
       for (int t = 0; t < 3; ++t) {
-        c.bin[t] = (int)std::min<int64_t>(want[t], n[t]);
+        c.bin[t] = want[t];
         c.tile[t] = c.bin[t] + c.taps - 1;
       }
       c.sparse = c.sparse_interp = 0;
@@ -678,7 +680,7 @@ int Engine::build_layout() {
       nb_total *= g.nbins[t];
       it.N[t] = t < s.d ? (int)s.N[t] : 1;
     }
-    g.fine = c.pencil ? c.bin[0] : 1;
+    g.fine = c.pencil ? std::min(c.bin[0], g.n[0]) : 1;
     it.NN = 1;
     for (int t = 0; t < s.d; ++t) it.NN *= s.N[t];
     it.M = s.M;
