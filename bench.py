@@ -213,9 +213,9 @@ def _traffic(workload, stage):
     return rec["bytes"]
 
 
-STAGE_KERNELS = {"spread": "k_spread_planes (dense bins) + k_spread_gm (sparse bins), after a grid memset",
-                 "interp": "k_interp_groups (dense bins) + k_interp_gm (sparse bins)",
-                 "sort": "k_bin_count + k_scan + k_scatter + subproblem kernels",
+STAGE_KERNELS = {"spread": "k_spread_pencil (pencil layout) or k_spread_planes + k_spread_gm (bins), after a grid memset",
+                 "interp": "k_interp_pencil (pencil layout) or k_interp_groups + k_interp_gm (bins)",
+                 "sort": "k_key_count + k_scan + k_scatter + subproblem kernels + k_refine (pencil layout)",
                  "fft": "cuFFT C2C", "ifft": "cuFFT C2C", "deconv": "k_deconv_crop", "pad": "k_pad_deconv"}
 
 
@@ -252,6 +252,8 @@ def _roofline(stages, workload, geom, peaks, kind, sms):
         # FMAs (4 flops) per update, against 128 FP32 lanes x 2 flops per clock per SM
         r["smem_pipe_" + st] = {"achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
                                 "peak_kind": "derived: %d SMs x 128 B/clk x %.0f MHz" % (sms, mhz),
+                                "note": "bytes of a shared-memory tile's cell updates (pencil spreading updates "
+                                        "registers; pencil interpolation of dense bins shares its reads)",
                                 "cell_updates_per_s": visits / ts,
                                 "alu_fp32_frac": visits * 4 / ts / (sms * 128 * 2 * mhz * 1e6)}
     return r

@@ -78,7 +78,10 @@ typedef enum {
 
 /* Spreading / interpolation kernels. */
 typedef enum {
-  NFFT_METHOD_AUTO = 0,   /* warp if available, else tiled if the tile fits, else global */
+  NFFT_METHOD_AUTO = 0,   /* warp if available, else tiled if the tile fits, else global;
+                             d = 3 in NFFT_FP32_MIXED with a point per pencil plane or
+                             more and no bin, split, owner or tensor-core option set:
+                             pencils (reported as NFFT_METHOD_WARP) */
   NFFT_METHOD_TILED = 1,  /* bin-sorted points, per-subproblem shared-memory tile */
   NFFT_METHOD_GLOBAL = 2, /* one thread per point, atomics straight into the grid
                              (the paper's spread kernel, Section 3) */
