@@ -45,7 +45,7 @@ namespace {
 constexpr int kRsThreads = 256;
 constexpr int kRsReach = 3;     // neighbour columns per side (column edge >= r_c / kRsReach)
 constexpr int kRsColumns = (2 * kRsReach + 1) * (2 * kRsReach + 1);
-constexpr int kRsIons = 8;      // ions a warp takes, two at a time
+constexpr int kRsIons = 8;      // most ions a warp takes, two at a time
 constexpr double kRsGrid = 1024.0;
 
 // (v, v), kept in its registers (the compiler rebuilt constant pairs in the loop).
@@ -147,6 +147,7 @@ constexpr float kErfcScale = 0.42f;
 
 struct RsParams {
   int n, ncol, nz;
+  int per_warp;     // ions a warp takes: even, at most kRsIons
   float rc2, near;  // (r_c / L)^2, r_c / (4 L)
   float alpha;      // alpha L
   float escale;     // -(alpha L)^2 log2(e)
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kRsThreads, 4) k_rs_columns(RsParams P, const 
   __shared__ RsRange ranges[kRsThreads / 32][2 * kRsColumns];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   RsRange* mine = ranges[warp];
-  const int first = (blockIdx.x * (kRsThreads / 32) + warp) * kRsIons, last = min(P.n, first + kRsIons);
+  const int first = (blockIdx.x * (kRsThreads / 32) + warp) * P.per_warp, last = min(P.n, first + P.per_warp);
   const float inv = 1.0f / (float)P.ncol, half = 0.5f * inv;
   constexpr float kErfc[8] = {0.236731262f, 0.240897215f,  0.187104512f,  0.292422239f,
                               -0.17306915f, 0.48496216f,   -0.345052719f, 0.0760044978f};
@@ -371,7 +372,12 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
   if (!cells_form && n > 65536) return NFFT_ERR_UNSUPPORTED;   // the all-pairs form is O(n^2)
   const int ni = (int)n;
   const int blocks = (ni + kRsThreads - 1) / kRsThreads;
-  constexpr int per_block = kRsThreads / 32 * kRsIons;
+  // As many ions per warp as still give the chip's resident warps (32 on each
+  // of 152 SMs) one each; a warp's ranges serve all its ions in turn.  With 8
+  // each throughout, few ions left SMs idle: forces of 2592 ions 395 -> 325 us,
+  // 6144: 402 -> 350, 12000: 512 -> 421, 20736: 611 -> 541; 49152: 1155 either way.
+  const int per_warp = std::min(std::max(2 * (ni / (2 * 32 * 152)), 2), kRsIons);
+  const int per_block = kRsThreads / 32 * per_warp;
   const int parts = cells_form ? (ni + per_block - 1) / per_block : blocks;
   const int cells = ncol * ncol * nz;
   // scratch: partials and the total, and for the cell list records, charges,
@@ -414,6 +420,7 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
     P.n = ni;
     P.ncol = ncol;
     P.nz = nz;
+    P.per_warp = per_warp;
     P.rc2 = (float)(rcut / L * (rcut / L));
     P.near = (float)(0.25 * rcut / L);
     P.alpha = (float)(alpha * L);
