@@ -43,3 +43,20 @@ def test_columns(n, L, rc, kind):
     assert np.abs(F.cpu().numpy() - want).max() <= 2e-5 * max(np.abs(want).max(), 1e-300)
     assert abs(got - e) <= 1e-6 * size
     assert abs(ewald_real_space(torch.from_numpy(r), torch.from_numpy(q), L, alpha, rc) - e) <= 1e-6 * size
+
+
+@pytest.mark.parametrize("n", [720, 721, 1081, 1443])
+def test_ions_per_warp(n):
+    """2, 4, 6 and 8 ions per warp: 27 copies of a box (a cube of 3 on a side) have its forces and 27 times its energy."""
+    from paper_2001_01583_gb300 import ewald_real_space_forces
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    L, rc, alpha = 9.0, 2.5, 0.8
+    r, q = _ions(n, L, "random", n)
+    want = ewald.real_space_forces(r, q, L, alpha, rc)
+    size = ewald.real_space_energy(r, np.abs(q), L, alpha, rc)
+    shifts = L * np.stack(np.meshgrid(*[np.arange(3.0)] * 3, indexing="ij"), -1).reshape(-1, 1, 3)
+    F, got = ewald_real_space_forces(torch.from_numpy((r + shifts).reshape(-1, 3)), torch.from_numpy(np.tile(q, 27)),
+                                     3 * L, alpha, rc)
+    assert np.abs(F.cpu().numpy().reshape(27, n, 3) - want).max() <= 2e-5 * np.abs(want).max()
+    assert abs(got - 27 * ewald.real_space_energy(r, q, L, alpha, rc)) <= 1e-6 * 27 * size
