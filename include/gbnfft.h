@@ -265,7 +265,9 @@ int nfft_ewald_reciprocal_sum(nfft_plan* plan, const void* S_dev, double L, doub
  * forward NFFT (Eq. 6) of three right-hand sides.  q_dev: M complex of the
  * plan's precision (real part = charge); F_dev: device, M x 3 doubles,
  * point-major, written asynchronously on the plan's stream.  The first call
- * allocates 3 |I_N| + 3 M complex values of scratch kept by the plan. */
+ * allocates 3 |I_N| + 3 M complex values of scratch kept by the plan, and
+ * with fewer than three grids (NFFT_OPT_RHS_CAPACITY) three of them where
+ * they are 64 MiB or less and there is memory; the plan's own grids stay. */
 int nfft_ewald_reciprocal_forces(nfft_plan* plan, const void* q_dev, double L, double alpha, double* F_dev);
 
 /* Largest |I_N| nfft_ewald_reciprocal_sum_noalloc accepts (4096 tiles of 8192). */

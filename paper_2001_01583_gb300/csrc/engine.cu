@@ -304,8 +304,7 @@ Engine::~Engine() {
   free_dev(err_flag);
   free_dev(ewald_partials);
   free_dev(ewald_out);
-  free_dev(force_modes);
-  free_dev(force_vals);
+  free_dev(force_buf);
   free_dev(d_items);
   for (int k = 0; k < 2; ++k) {
     if (h_table[k]) cudaFreeHost(h_table[k]);
@@ -912,7 +911,8 @@ int Engine::build_pruned(FClass& fc) {
   return NFFT_OK;
 }
 
-int Engine::run_fft(FClass& fc, int batch, int64_t grid_offset, int direction) {
+// `batch` grids of the class's shape, one after another from `grids`.
+int Engine::run_fft(FClass& fc, int batch, void* grids, int direction) {
   if (fft_pruned(fc)) {
     TRY(build_pruned(fc));
     if (cufftSetStream(fc.prune_z, stream) != CUFFT_SUCCESS || cufftSetStream(fc.prune_yx, stream) != CUFFT_SUCCESS)
@@ -920,15 +920,15 @@ int Engine::run_fft(FClass& fc, int batch, int64_t grid_offset, int direction) {
     const int64_t plane = fc.n[1] * fc.n[2];
     const int64_t upper = (fc.n[0] - items[0].N[0] / 2) * plane;   // first plane of the k < 0 run
     for (int b = 0; b < batch; ++b) {
-      const int64_t g0 = grid_offset + (int64_t)b * fc.cells;
+      const int64_t g0 = (int64_t)b * fc.cells;
       cufftResult r = CUFFT_SUCCESS;
       auto exec = [&](cufftHandle h, int64_t off) {
         if (r != CUFFT_SUCCESS) return;
         if (precision == NFFT_FP64) {
-          cufftDoubleComplex* g = static_cast<cufftDoubleComplex*>(fc.buf) + off;
+          cufftDoubleComplex* g = static_cast<cufftDoubleComplex*>(grids) + off;
           r = cufftExecZ2Z(h, g, g, direction);
         } else {
-          cufftComplex* g = static_cast<cufftComplex*>(fc.buf) + off;
+          cufftComplex* g = static_cast<cufftComplex*>(grids) + off;
           r = cufftExecC2C(h, g, g, direction);
         }
       };
@@ -949,10 +949,10 @@ int Engine::run_fft(FClass& fc, int batch, int64_t grid_offset, int direction) {
   TRY(fft_handle(fc, batch, &h));
   cufftResult r;
   if (precision == NFFT_FP64) {
-    cufftDoubleComplex* g = static_cast<cufftDoubleComplex*>(fc.buf) + grid_offset;
+    cufftDoubleComplex* g = static_cast<cufftDoubleComplex*>(grids);
     r = cufftExecZ2Z(h, g, g, direction);
   } else {
-    cufftComplex* g = static_cast<cufftComplex*>(fc.buf) + grid_offset;
+    cufftComplex* g = static_cast<cufftComplex*>(grids);
     r = cufftExecC2C(h, g, g, direction);
   }
   return r == CUFFT_SUCCESS ? NFFT_OK : NFFT_ERR_CUFFT;
@@ -1025,7 +1025,7 @@ int Engine::blocks_per_sm(const void* fn, int threads, size_t smem) {
 // point kernels
 
 template <typename Real>
-int Engine::run_points(const KClass& kc, bool spread, const void* in, void* out, int nrhs) {
+int Engine::run_points(const KClass& kc, bool spread, const void* in, void* out, int nrhs, const ItemDev* table) {
   PointKernelArgs<Real> a{};
   a.pts.perm = perm;
   a.pts.local = local;
@@ -1035,7 +1035,7 @@ int Engine::run_points(const KClass& kc, bool spread, const void* in, void* out,
   a.pts.num_subs = num_subs;
   a.pts.bin_count = bin_count;
   a.pts.bin_start = bin_start;
-  a.items = d_items;
+  a.items = table ? table : d_items;
   a.item_begin = kc.item_begin;
   a.item_end = kc.item_end;
   a.bin_begin = kc.bin_begin;
@@ -1402,7 +1402,7 @@ int Engine::adjoint_single(const void* f, void* fhat, int R) {
       TRY(stage_end(&ev));
       continue;
     }
-    TRY(run_fft(fc, nr, item_grid_offset[0], CUFFT_FORWARD));
+    TRY(run_fft(fc, nr, it.grid, CUFFT_FORWARD));
     TRY(stage_end(&ev));
     TRY(stage_begin(NFFT_STAGE_DECONV, &ev));
     const int64_t cblocks = scale_blocks(it.NN / it.N[it.geom.d - 1] * nr, it.N[it.geom.d - 1], false);
@@ -1414,43 +1414,46 @@ int Engine::adjoint_single(const void* f, void* fhat, int R) {
   return NFFT_OK;
 }
 
-int Engine::forward_single(const void* fhat, void* f, int R, int cap) {
-  FClass& fc = fclasses[item_fclass[0]];
+int Engine::forward_single(const void* fhat, void* f, int R) {
   const ItemDev& it = items[0];
-  if (cap < rhs_cap) cap = rhs_cap;
-  for (int r0 = 0; r0 < R; r0 += cap) {
-    const int nr = (R - r0) < cap ? (R - r0) : cap;
-    EventPair ev{};
-    const void* hin = static_cast<const char*>(fhat) + (int64_t)r0 * it.NN * (int64_t)csize;
-    if (direct_dft(fc, nr)) {
-      TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
-      CK(launch_pad_dft(d_items, fc.roots, (int)fc.n[0], hin, nr, stream));
-      ++kernel_launches;
-      TRY(stage_end(&ev));
-    } else {
-      TRY(stage_begin(NFFT_STAGE_PAD, &ev));
-      const int64_t pblocks = scale_blocks(fc.cells / fc.n[fc.d - 1] * nr, fc.n[fc.d - 1], false);
-      CK(precision == NFFT_FP64 ? launch_pad_deconv<double>(d_items, nullptr, nullptr, pblocks, hin, nr, stream)
-                                : launch_pad_deconv<float>(d_items, nullptr, nullptr, pblocks, hin, nr, stream));
-      kernel_launches += pblocks > 0 ? 1 : 0;
-      TRY(stage_end(&ev));
-      TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
-      if (nr <= rhs_cap) {
-        TRY(run_fft(fc, nr, item_grid_offset[0], CUFFT_INVERSE));
-      } else {   // more grids than the plan's transforms take at once
-        for (int b = 0; b < nr; ++b) TRY(run_fft(fc, 1, item_grid_offset[0] + b * fc.cells, CUFFT_INVERSE));
-      }
-      TRY(stage_end(&ev));
-    }
-    TRY(stage_begin(NFFT_STAGE_INTERP, &ev));
-    if (it.M > 0) {
-      void* fout = static_cast<char*>(f) + (int64_t)r0 * it.M * (int64_t)csize;
-      // interpolation reads `in` only through the override flag; the values come from the grid
-      TRY(precision == NFFT_FP64 ? run_points<double>(kclasses[0], false, fout, fout, nr)
-                                 : run_points<float>(kclasses[0], false, fout, fout, nr));
-    }
+  for (int r0 = 0; r0 < R; r0 += rhs_cap) {
+    const int nr = (R - r0) < rhs_cap ? (R - r0) : rhs_cap;
+    TRY(forward_grids(d_items, it.grid, nr, static_cast<const char*>(fhat) + (int64_t)r0 * it.NN * (int64_t)csize,
+                      static_cast<char*>(f) + (int64_t)r0 * it.M * (int64_t)csize, nr));
+  }
+  return NFFT_OK;
+}
+
+// nr right-hand sides on nr grids: `item` is the plan's item on the device with
+// its grid at `grids`; fft_batch of them are transformed at once.
+int Engine::forward_grids(const ItemDev* item, void* grids, int fft_batch, const void* fhat, void* f, int nr) {
+  FClass& fc = fclasses[item_fclass[0]];
+  EventPair ev{};
+  if (direct_dft(fc, nr)) {
+    TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
+    CK(launch_pad_dft(item, fc.roots, (int)fc.n[0], fhat, nr, stream));
+    ++kernel_launches;
+    TRY(stage_end(&ev));
+  } else {
+    TRY(stage_begin(NFFT_STAGE_PAD, &ev));
+    const int64_t pblocks = scale_blocks(fc.cells / fc.n[fc.d - 1] * nr, fc.n[fc.d - 1], false);
+    CK(precision == NFFT_FP64 ? launch_pad_deconv<double>(item, nullptr, nullptr, pblocks, fhat, nr, stream)
+                              : launch_pad_deconv<float>(item, nullptr, nullptr, pblocks, fhat, nr, stream));
+    kernel_launches += pblocks > 0 ? 1 : 0;
+    TRY(stage_end(&ev));
+    TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
+    for (int b = 0; b < nr; b += fft_batch)
+      TRY(run_fft(fc, std::min(fft_batch, nr - b), static_cast<char*>(grids) + (int64_t)b * fc.cells * (int64_t)csize,
+                  CUFFT_INVERSE));
     TRY(stage_end(&ev));
   }
+  TRY(stage_begin(NFFT_STAGE_INTERP, &ev));
+  if (items[0].M > 0) {
+    // interpolation reads `in` only through the override flag; the values come from the grid
+    TRY(precision == NFFT_FP64 ? run_points<double>(kclasses[0], false, f, f, nr, item)
+                               : run_points<float>(kclasses[0], false, f, f, nr, item));
+  }
+  TRY(stage_end(&ev));
   return NFFT_OK;
 }
 
@@ -1466,7 +1469,7 @@ int Engine::adjoint_table(bool in_graph) {
   for (const auto& kc : kclasses) TRY(run_points<Real>(kc, true, nullptr, nullptr, 0));
   if (!in_graph) TRY(stage_end(&ev));
   if (!in_graph) TRY(stage_begin(NFFT_STAGE_FFT, &ev));
-  for (auto& fc : fclasses) TRY(run_fft(fc, fc.grids, 0, CUFFT_FORWARD));
+  for (auto& fc : fclasses) TRY(run_fft(fc, fc.grids, fc.buf, CUFFT_FORWARD));
   if (!in_graph) TRY(stage_end(&ev));
   if (!in_graph) TRY(stage_begin(NFFT_STAGE_DECONV, &ev));
   CK(launch_deconv_crop<Real>(d_items, d_crop_blocks, d_crop_blocks + items.size() + 1, crop_blocks, nullptr, 0,
@@ -1485,7 +1488,7 @@ int Engine::forward_table(bool in_graph) {
   kernel_launches += pad_blocks > 0 ? 1 : 0;
   if (!in_graph) TRY(stage_end(&ev));
   if (!in_graph) TRY(stage_begin(NFFT_STAGE_IFFT, &ev));
-  for (auto& fc : fclasses) TRY(run_fft(fc, fc.grids, 0, CUFFT_INVERSE));
+  for (auto& fc : fclasses) TRY(run_fft(fc, fc.grids, fc.buf, CUFFT_INVERSE));
   if (!in_graph) TRY(stage_end(&ev));
   if (!in_graph) TRY(stage_begin(NFFT_STAGE_INTERP, &ev));
   for (const auto& kc : kclasses) TRY(run_points<Real>(kc, false, nullptr, nullptr, 0));
@@ -1599,7 +1602,7 @@ int Engine::ewald_impl(const void* q, double L, double alpha) {
   if (it.M > 0) TRY(run_points<Real>(kclasses[0], true, q, nullptr, 1));
   TRY(stage_end(&ev));
   TRY(stage_begin(NFFT_STAGE_FFT, &ev));
-  TRY(run_fft(fc, 1, item_grid_offset[0], CUFFT_FORWARD));
+  TRY(run_fft(fc, 1, it.grid, CUFFT_FORWARD));
   TRY(stage_end(&ev));
   TRY(stage_begin(NFFT_STAGE_DECONV, &ev));
   EwaldGeom g{};
@@ -1640,37 +1643,37 @@ int Engine::ewald(const void* q, double L, double alpha, double* out) {
 // one after another otherwise or when there is no memory for more.
 constexpr size_t kForceGridBytes = (size_t)64 << 20;
 
-int Engine::force_grids() {
-  FClass& fc = fclasses[item_fclass[0]];
-  const size_t one = (size_t)fc.cells * csize;
-  if (fc.grids >= 3) return 3;
-  if (3 * one > kForceGridBytes) return rhs_cap;
-  void* grown = nullptr;
-  if (alloc_dev(grown, 3 * one, device_bytes) != NFFT_OK) return rhs_cap;
-  // queued work still uses the old grids
-  if (cudaStreamSynchronize(stream) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(grown);
-    device_bytes -= (int64_t)(3 * one);
-    return rhs_cap;
+// The forces' own buffer, allocated by the first call: modes, values, the
+// three grids and the item that points at them.  The plan's grid stays where
+// it is: graphs captured from other calls hold its address.
+int Engine::force_alloc() {
+  if (force_buf) return NFFT_OK;
+  const ItemDev& it = items[0];
+  auto part = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+  const size_t modes = part((size_t)3 * (size_t)it.NN * csize), vals = part((size_t)3 * (size_t)it.M * csize);
+  const size_t grids = (size_t)3 * (size_t)it.geom.grid_cells * csize;
+  const bool together = rhs_cap < 3 && grids <= kForceGridBytes;
+  char* p = nullptr;
+  int st = NFFT_ERR_OOM;
+  if (together) st = alloc_dev(p, modes + vals + part(sizeof(ItemDev)) + grids, device_bytes);
+  if (st == NFFT_OK) {
+    force_item = reinterpret_cast<ItemDev*>(p + modes + vals);
+    force_grids = p + modes + vals + part(sizeof(ItemDev));
+  } else {
+    TRY(alloc_dev(p, modes + vals, device_bytes));
   }
-  free_dev(fc.buf);
-  device_bytes -= (int64_t)((size_t)fc.grids * one);
-  fc.buf = grown;
-  fc.grids = 3;
-  items[0].grid = grown;
-  // a failure here shows in every later call on the stream
-  cudaMemcpyAsync(d_items, items.data(), sizeof(ItemDev), cudaMemcpyHostToDevice, stream);
-  return 3;
+  force_buf = p;
+  force_modes = p;
+  force_vals = p + modes;
+  return NFFT_OK;
 }
 
 template <typename Real>
 int Engine::ewald_forces_impl(const void* q, double L, double alpha, double* F) {
   using C = typename Cplx<Real>::type;
   const ItemDev& it = items[0];
-  if (!force_modes) TRY(alloc_dev(force_modes, (size_t)3 * (size_t)it.NN * csize, device_bytes));
-  if (!force_vals && it.M > 0) TRY(alloc_dev(force_vals, (size_t)3 * (size_t)it.M * csize, device_bytes));
-  const int cap = force_grids();
+  TRY(force_alloc());
+  const bool together = force_grids && rhs_cap < 3;
   // S(n): the adjoint NFFT (Eq. 5) of the charges, into the first block
   TRY(adjoint_single(q, force_modes, 1));
   EwaldGeom g{};
@@ -1683,11 +1686,15 @@ int Engine::ewald_forces_impl(const void* q, double L, double alpha, double* F) 
   }
   const double al = alpha * L;
   g.coef = M_PI * M_PI / (al * al);
-  CK(launch_force_modes<Real>(static_cast<C*>(force_modes), g, stream));
+  CK(launch_force_modes<Real>(static_cast<C*>(force_modes), g, d_items, together ? force_item : nullptr, force_grids,
+                              stream));
   kernel_launches += it.NN > 0 ? 1 : 0;
   if (it.M == 0) return NFFT_OK;
   // sum_n w(n) n_t S(n) exp(+2 pi i n.x_i): the forward NFFT (Eq. 6), three right-hand sides
-  TRY(forward_single(force_modes, force_vals, 3, cap));
+  if (together)
+    TRY(forward_grids(force_item, force_grids, rhs_cap, force_modes, force_vals, 3));
+  else
+    TRY(forward_single(force_modes, force_vals, 3));
   CK(launch_force_finish<Real>(static_cast<const C*>(force_vals), static_cast<const C*>(q), it.M, 2.0 / (L * L), F,
                                stream));
   kernel_launches += 1;

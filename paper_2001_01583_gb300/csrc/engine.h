@@ -92,7 +92,7 @@ class Engine {
   int set_points_single(const double* x);
   int set_points_batch(const double* const* x);
   int adjoint_single(const void* f, void* fhat, int R);
-  int forward_single(const void* fhat, void* f, int R, int cap = 0);   // cap: grids to use at once (at least rhs_cap)
+  int forward_single(const void* fhat, void* f, int R);
   int adjoint_batch(const void* const* f, void* const* fhat);
   int forward_batch(const void* const* fhat, void* const* f);
   int sync();
@@ -120,7 +120,9 @@ class Engine {
   int release_layout();
   int build_fft();
   template <typename Real> int set_points_impl(const double* x_override);
-  template <typename Real> int run_points(const KClass& kc, bool spread, const void* in, void* out, int nrhs);
+  // table: the items on the device (null: d_items)
+  template <typename Real>
+  int run_points(const KClass& kc, bool spread, const void* in, void* out, int nrhs, const ItemDev* table = nullptr);
   template <typename Real> int run_planes(const KClass& kc, PointKernelArgs<Real>& a, bool spread, int max_nrhs);
   template <typename Real> int run_wpp(const KClass& kc, PointKernelArgs<Real>& a, bool spread, int max_nrhs);
   template <typename Real> int run_tiled(const KClass& kc, PointKernelArgs<Real>& a, bool spread, int max_nrhs);
@@ -133,12 +135,13 @@ class Engine {
   template <typename Real> int forward_table(bool in_graph);
   template <typename Real> int ewald_impl(const void* q, double L, double alpha);
   template <typename Real> int ewald_forces_impl(const void* q, double L, double alpha, double* F);
-  int run_fft(FClass& fc, int batch, int64_t grid_offset, int direction);
+  int run_fft(FClass& fc, int batch, void* grids, int direction);
+  int forward_grids(const ItemDev* item, void* grids, int fft_batch, const void* fhat, void* f, int nr);
   bool fft_pruned(const FClass& fc) const;
   bool direct_dft(const FClass& fc, int nr) const;
   int build_pruned(FClass& fc);
   void destroy_fft_plans(FClass& fc);
-  int force_grids();
+  int force_alloc();
   int fft_handle(FClass& fc, int batch, cufftHandle* out);
   int blocks_per_sm(const void* fn, int threads, size_t smem);
   int stage_begin(int stage, EventPair* ev);
@@ -216,8 +219,12 @@ class Engine {
   int* err_flag = nullptr;
   double* ewald_partials = nullptr;
   double* ewald_out = nullptr;
-  void* force_modes = nullptr;   // 3 |I_N| complex (forces)
-  void* force_vals = nullptr;    // 3 M complex (forces)
+  // forces: one allocation of the first call, and its parts
+  char* force_buf = nullptr;
+  void* force_modes = nullptr;      // 3 |I_N| complex
+  void* force_vals = nullptr;       // 3 M complex
+  ItemDev* force_item = nullptr;    // the plan's item with its grid at force_grids (written by every call)
+  void* force_grids = nullptr;      // three grids, or null: the plan's
   int64_t device_bytes = 0;
   int64_t layout_bytes = 0;
 

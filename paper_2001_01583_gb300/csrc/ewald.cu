@@ -163,10 +163,17 @@ __global__ void __launch_bounds__(kThreads) k_finish(const double* __restrict__ 
 }
 
 // w(n) n_t S(n) for t = 0, 1, 2 from S in block 0 (each thread reads its
-// S(n) before writing the three blocks at the same index).
+// S(n) before writing the three blocks at the same index).  item_out: a copy
+// of *item with its grid at `grids` (null: none).
 template <typename Real>
-__global__ void __launch_bounds__(kThreads) k_force_modes(typename Cplx<Real>::type* __restrict__ modes, EwaldGeom g) {
+__global__ void __launch_bounds__(kThreads) k_force_modes(typename Cplx<Real>::type* __restrict__ modes, EwaldGeom g,
+                                                          const ItemDev* __restrict__ item, ItemDev* item_out,
+                                                          void* grids) {
   using C = typename Cplx<Real>::type;
+  if (item_out && blockIdx.x == 0 && threadIdx.x == 0) {
+    *item_out = *item;
+    item_out->grid = grids;
+  }
   __shared__ double tab[kEwaldTabMax];
   const double* tp = ewald_tables(g, tab) ? tab : nullptr;
   for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < g.NN; e += (int64_t)gridDim.x * kThreads) {
@@ -196,10 +203,11 @@ __global__ void __launch_bounds__(kThreads) k_force_finish(const typename Cplx<R
 }  // namespace
 
 template <typename Real>
-cudaError_t launch_force_modes(typename Cplx<Real>::type* modes, const EwaldGeom& g, cudaStream_t st) {
+cudaError_t launch_force_modes(typename Cplx<Real>::type* modes, const EwaldGeom& g, const ItemDev* item,
+                               ItemDev* item_out, void* grids, cudaStream_t st) {
   if (g.NN == 0) return cudaSuccess;
   const int64_t blocks = std::min<int64_t>((g.NN + kThreads - 1) / kThreads, 65535);
-  k_force_modes<Real><<<(unsigned)blocks, kThreads, 0, st>>>(modes, g);
+  k_force_modes<Real><<<(unsigned)blocks, kThreads, 0, st>>>(modes, g, item, item_out, grids);
   return cudaGetLastError();
 }
 
@@ -212,8 +220,8 @@ cudaError_t launch_force_finish(const typename Cplx<Real>::type* vals, const typ
   return cudaGetLastError();
 }
 
-template cudaError_t launch_force_modes<float>(float2*, const EwaldGeom&, cudaStream_t);
-template cudaError_t launch_force_modes<double>(double2*, const EwaldGeom&, cudaStream_t);
+template cudaError_t launch_force_modes<float>(float2*, const EwaldGeom&, const ItemDev*, ItemDev*, void*, cudaStream_t);
+template cudaError_t launch_force_modes<double>(double2*, const EwaldGeom&, const ItemDev*, ItemDev*, void*, cudaStream_t);
 template cudaError_t launch_force_finish<float>(const float2*, const float2*, int64_t, double, double*, cudaStream_t);
 template cudaError_t launch_force_finish<double>(const double2*, const double2*, int64_t, double, double*,
                                                  cudaStream_t);

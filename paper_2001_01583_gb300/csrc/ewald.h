@@ -32,8 +32,10 @@ cudaError_t launch_ewald_sum(const typename Cplx<Real>::type* src, bool from_gri
 // (C order) in its first |I_N| complex values; afterwards its three blocks of
 // |I_N| hold w(n) n_t S(n), t = 0, 1, 2, w(n) = exp(-coef |n|^2) / |n|^2
 // (0 at n = 0), the right-hand sides of a forward NFFT (Eq. 6).  Requires d = 3.
+// item_out (may be null): gets *item with its grid at `grids`.
 template <typename Real>
-cudaError_t launch_force_modes(typename Cplx<Real>::type* modes, const EwaldGeom& g, cudaStream_t st);
+cudaError_t launch_force_modes(typename Cplx<Real>::type* modes, const EwaldGeom& g, const ItemDev* item,
+                               ItemDev* item_out, void* grids, cudaStream_t st);
 // F[i][t] = scale * Re(q_i) * Im(vals[t][i]) for i < M, t < 3 (vals: three
 // blocks of M complex, the forward NFFT of the force modes at the points).
 template <typename Real>
