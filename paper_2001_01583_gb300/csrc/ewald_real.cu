@@ -22,7 +22,8 @@
 //     and y are FP32 offsets from its column's axis, its z the sum of a
 //     multiple of 2^-10 and an FP32 remainder, so that separations carry an
 //     error of about 1e-9 L and neither box coordinates nor periodic shifts
-//     are rounded; pair terms and a lane's sums are FP32;
+//     are rounded; pair terms and the sums over a range are FP32, an ion's sums
+//     over its ranges FP64;
 //   - all pairs (smaller boxes): the minimum image of every pair plus the 26
 //     shifts by L, all in FP64, which is the definition itself (r_c < L).
 // The energy 1/2 sum_i q_i phi_i is reduced in FP64 in a fixed order (block
@@ -247,12 +248,11 @@ __global__ void __launch_bounds__(kRsThreads, 4) k_rs_columns(RsParams P, const 
       }
     }
     __syncwarp();
-    Pair phi = 0, fx = 0, fy = 0, fz = 0;
+    double sum = 0.0;   // lane l: its share of value l >> 2 of (phi, f) of the first ion, then of the second
     for (int k = 0; k < count; ++k) {
       const RsRange rg = mine[k];
       const float sxa = rg.dx - pa.x, sxb = rg.dx - pb.x, sya = rg.dy - pa.y, syb = rg.dy - pb.y;
-      // a range's sums on their own first: shorter FP32 sums
-      Pair rphi = 0, rfx = 0, rfy = 0, rfz = 0;
+      Pair phi = 0, fx = 0, fy = 0, fz = 0;   // a range's sums: FP32, over its lanes too; FP64 over the ranges
       const float sha = rg.dz - pa.z, shb = rg.dz - pb.z, sla = -pa.w, slb = -pb.w;
 #pragma unroll 2
       for (int j0 = rg.begin; j0 < rg.end; j0 += 32) {
@@ -272,28 +272,31 @@ __global__ void __launch_bounds__(kRsThreads, 4) k_rs_columns(RsParams P, const 
         for (int c = 6; c >= 0; --c) w = pair_fma(w, t, cf[c]);
         const Pair q2 = pair(qa, qb);
         const Pair ec = pair_mul(pair_mul(pair_mul(w, t), ee), rinv);   // erfc(alpha r) / r
-        rphi = pair_fma(q2, ec, rphi);
+        phi = pair_fma(q2, ec, phi);
         if (FORCES) {
           const Pair g = pair_mul(pair_mul(pair_fma(ee, c2, ec), pair_mul(rinv, rinv)), q2);
-          rfx = pair_fma(g, X, rfx);
-          rfy = pair_fma(g, Y, rfy);
-          rfz = pair_fma(g, Z, rfz);
+          fx = pair_fma(g, X, fx);
+          fy = pair_fma(g, Y, fy);
+          fz = pair_fma(g, Z, fz);
         }
       }
-      phi = pair_add(phi, rphi);
-      fx = pair_add(fx, rfx);
-      fy = pair_add(fy, rfy);
-      fz = pair_add(fz, rfz);
+      const float2 p2 = halves(phi);
+      if (FORCES) {
+        const float2 x2 = halves(fx), y2 = halves(fy), z2 = halves(fz);
+        const float v[8] = {p2.x, x2.x, y2.x, z2.x, p2.y, x2.y, y2.y, z2.y};
+        sum += (double)butterfly8_shares(v, lane);
+      } else {
+        const bool second = lane >= 16;
+        sum += (double)((second ? p2.y : p2.x) + __shfl_xor_sync(0xffffffffu, second ? p2.x : p2.y, 16));
+      }
     }
-    // over the warp: lane l gets value l >> 2 of (phi, f) of the first ion, then of the second
-    const float2 p2 = halves(phi), x2 = halves(fx), y2 = halves(fy), z2 = halves(fz);
-    const float v[8] = {p2.x, x2.x, y2.x, z2.x, p2.y, x2.y, y2.y, z2.y};
-    const float sum = butterfly8(v, lane);
+#pragma unroll
+    for (int o = FORCES ? 2 : 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     const int which = lane >> 4, comp = (lane >> 2) & 3;
     if ((lane & 3) == 0 && (which == 0 || two)) {
       const double qi = (double)rec_q[i + which];
-      if (comp == 0) e += qi * (double)sum * P.phi_scale;
-      else if (FORCES) F[(int64_t)rec_idx[i + which] * 3 + comp - 1] = -qi * (double)sum * P.f_scale;
+      if (comp == 0) e += qi * sum * P.phi_scale;
+      else if (FORCES) F[(int64_t)rec_idx[i + which] * 3 + comp - 1] = -qi * sum * P.f_scale;
     }
     i += two ? 2 : 1;
   }

@@ -35,11 +35,10 @@ __device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
   return d;
 }
 
-// Eight values reduced over the warp at once by a transposed butterfly (9
-// shuffles): after the exchanges over lane bits 4, 3 and 2 each
-// lane keeps one value, and bits 1 and 0 finish its sum.  Lane l returns the
-// sum of value l >> 2.
-__device__ __forceinline__ float butterfly8(const float* v, int lane) {
+// Eight values reduced over the warp at once by a transposed butterfly (7
+// shuffles): after the exchanges over lane bits 4, 3 and 2 lane l keeps its
+// share of value l >> 2; the four lanes of a value have its sum between them.
+__device__ __forceinline__ float butterfly8_shares(const float* v, int lane) {
   const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
   float a4[4], a2[2];
 #pragma unroll
@@ -54,12 +53,13 @@ __device__ __forceinline__ float butterfly8(const float* v, int lane) {
     const float keep = b3 ? a4[2 + j] : a4[j];
     a2[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
   }
-  float a1;
-  {
-    const float send = b2 ? a2[0] : a2[1];
-    const float keep = b2 ? a2[1] : a2[0];
-    a1 = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
+  const float send = b2 ? a2[0] : a2[1];
+  const float keep = b2 ? a2[1] : a2[0];
+  return keep + __shfl_xor_sync(0xffffffffu, send, 4);
+}
+// The same with the shares added up (9 shuffles): lane l returns the sum of value l >> 2.
+__device__ __forceinline__ float butterfly8(const float* v, int lane) {
+  float a1 = butterfly8_shares(v, lane);
   a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
   a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
   return a1;
