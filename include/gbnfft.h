@@ -305,8 +305,11 @@ int nfft_ewald_reciprocal_sum_noalloc(int d, const int64_t* N, int precision, co
  * each visits the parts within rcut of the 7^2 columns around its own (only
  * the minimum image of a pair is within rcut); the pair terms are FP32 from
  * offsets to the columns' axes, summed in FP32 over a column's part and in
- * FP64 per ion.  Otherwise every pair and its 27 nearest images are summed in
- * FP64 (n <= 65536, else NFFT_ERR_UNSUPPORTED).  The total is a fixed-order FP64 reduction.
+ * FP64 per ion.  Many ions with few partners (fewer than 500 on average) are
+ * sorted into cells of edge >= rcut / 2 instead, and each visits the 5^3 cells
+ * around its own, with FP32 pair terms from offsets to the cells' centres and
+ * FP64 sums per ion.  Otherwise every pair and its 27 nearest images are
+ * summed in FP64 (n <= 65536, else NFFT_ERR_UNSUPPORTED).  The total is a fixed-order FP64 reduction.
  * Allocates scratch, runs on cuda_stream (NULL = legacy default stream) and
  * waits for it; *energy gets U^R (host double).  The paper computes this term
  * on the CPU side of its method; the library adds it so that the whole
@@ -318,8 +321,8 @@ int nfft_ewald_real_space(int64_t n, const double* r_dev, const double* q_dev, d
  * formula in the paper, the derivative written out):
  *   F_i = q_i sum_j q_j (erfc(alpha d)/d + 2 alpha/sqrt(pi) exp(-alpha^2 d^2)) (r_i - r_j + n L) / d^2
  * over the pairs and images with d = |r_i - r_j + n L| < rcut, by the same
- * two forms as nfft_ewald_real_space (columns with FP32 pair terms and FP64
- * sums per ion, or all pairs in FP64).  F_dev: device, n x 3 doubles in the
+ * forms as nfft_ewald_real_space (columns or cells with FP32 pair terms and
+ * FP64 sums per ion, or all pairs in FP64).  F_dev: device, n x 3 doubles in the
  * input order; *energy gets U^R as nfft_ewald_real_space would.  Allocates
  * scratch, runs on cuda_stream and waits for it. */
 int nfft_ewald_real_space_forces(int64_t n, const double* r_dev, const double* q_dev, double L, double alpha,

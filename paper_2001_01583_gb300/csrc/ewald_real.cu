@@ -45,8 +45,17 @@ namespace {
 
 constexpr int kRsThreads = 256;
 constexpr int kRsReach = 3;     // neighbour columns per side (column edge >= r_c / kRsReach)
+constexpr int kRsCellReach = 2; // neighbour cells per side (cell edge >= r_c / kRsCellReach)
 constexpr int kRsColumns = (2 * kRsReach + 1) * (2 * kRsReach + 1);
 constexpr int kRsIons = 8;      // most ions a warp takes, two at a time
+// Partners per ion (on average) below which the cells are taken: 500, and
+// fewer where the ions do not fill the chip with threads (x ions per SM).  The
+// cells' time is then the latency of one thread, about 345 + 0.92 us per
+// partner, that of the columns about 300 + 1.27 x.  Forces, uniform ions, cells /
+// columns: 36,000 ions and 120 partners 480 / 583 us, 300: 638 / 600; 165,888 ions
+// and 60: 712 / 1264, 500: 1322 / 1244; 393,216 ions and 60: 1181 / 2485, 400: 2025
+// / 2361, 1000: 3742 / 2630.
+inline double cell_partners(double ions_per_sm) { return std::min(500.0, 1.4 * ions_per_sm - 50.0); }
 constexpr double kRsGrid = 1024.0;
 
 // (v, v), kept in its registers (the compiler rebuilt constant pairs in the loop).
@@ -106,7 +115,7 @@ __device__ __forceinline__ double rs_fraction(double r, double L) {
 }
 __device__ __forceinline__ int rs_cell(double s, int n) { return min((int)(s * n), n - 1); }
 
-// (Column, z bin) of each ion and its rank there.
+// (Column, z bin) of each ion and its rank there (cells: ncol = nz).
 __global__ void k_rs_count(int64_t n, const double* __restrict__ r, double L, int ncol, int nz, int* __restrict__ count,
                            int2* __restrict__ cell_rank) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -138,7 +147,92 @@ __global__ void k_rs_scatter(int64_t n, const double* __restrict__ r, const doub
   if (rec_idx) rec_idx[p] = (int)i;
 }
 
+// The same for cells: offsets from the cell's centre and the charge.
+__global__ void k_rs_scatter_cells(int64_t n, const double* __restrict__ r, const double* __restrict__ q, double L,
+                                   int nc, const int* __restrict__ start, const int2* __restrict__ cell_rank,
+                                   float4* __restrict__ rec, int* __restrict__ rec_cell, int* __restrict__ rec_idx) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int2 cr = cell_rank[i];
+  const int cc[3] = {cr.x / (nc * nc), cr.x / nc % nc, cr.x % nc};
+  const double h = L / nc;
+  float o[3];
+  bool placed = true;
+  for (int t = 0; t < 3; ++t) {
+    const double x = r[i * 3 + t];
+    placed = placed && isfinite(x);
+    o[t] = (float)(rs_fraction(x, L) * L - (cc[t] + 0.5) * h);
+  }
+  const int p = start[cr.x] + cr.y;
+  rec[p] = make_float4(o[0], o[1], o[2], placed ? (float)q[i] : 0.f);
+  rec_cell[p] = cr.x;
+  if (rec_idx) rec_idx[p] = (int)i;
+}
+
+constexpr float kTwoOverSqrtPiF = 1.1283791670955126f;
 constexpr double kTwoOverSqrtPi = 1.1283791670955126;
+
+// Few partners: a thread per sorted ion over the cells around its own; block
+// partials of q_i phi_i.  FORCES: also the ion's force, written to its
+// original index (F: n x 3 doubles).
+template <bool FORCES>
+__global__ void __launch_bounds__(kRsThreads) k_rs_cells(int n, int nc, float h, float rc2, float alpha,
+                                                         const float4* __restrict__ rec,
+                                                         const int* __restrict__ rec_cell,
+                                                         const int* __restrict__ start, double* __restrict__ partial,
+                                                         const int* __restrict__ rec_idx, double* __restrict__ F) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double e = 0.0;
+  if (i < n) {
+    const float4 pi = rec[i];
+    const int cell = rec_cell[i];
+    const int cz = cell % nc, cy = cell / nc % nc, cx = cell / (nc * nc);
+    double phi = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
+    const float c2 = kTwoOverSqrtPiF * alpha, a2 = alpha * alpha;
+    for (int dx = -kRsCellReach; dx <= kRsCellReach; ++dx) {
+      const int x = cx + dx < 0 ? cx + dx + nc : (cx + dx >= nc ? cx + dx - nc : cx + dx);
+      for (int dy = -kRsCellReach; dy <= kRsCellReach; ++dy) {
+        const int y = cy + dy < 0 ? cy + dy + nc : (cy + dy >= nc ? cy + dy - nc : cy + dy);
+        for (int dz = -kRsCellReach; dz <= kRsCellReach; ++dz) {
+          const int z = cz + dz < 0 ? cz + dz + nc : (cz + dz >= nc ? cz + dz - nc : cz + dz);
+          const int nb = (x * nc + y) * nc + z;
+          const float sx = dx * h - pi.x, sy = dy * h - pi.y, sz = dz * h - pi.z;
+          float acc = 0.0f, ax = 0.0f, ay = 0.0f, az = 0.0f;
+          for (int j = start[nb]; j < start[nb + 1]; ++j) {
+            const float4 pj = rec[j];
+            const float rx = pj.x + sx, ry = pj.y + sy, rz = pj.z + sz;   // r_j - r_i
+            const float d2 = rx * rx + ry * ry + rz * rz;
+            if (d2 < rc2 && d2 > 0.0f) {
+              const float rinv = rsqrtf(d2);
+              const float ec = erfcf(alpha * d2 * rinv) * rinv;
+              acc += pj.w * ec;
+              if (FORCES) {
+                const float g = pj.w * (ec + c2 * __expf(-a2 * d2)) * rinv * rinv;
+                ax -= g * rx;
+                ay -= g * ry;
+                az -= g * rz;
+              }
+            }
+          }
+          phi += (double)acc;
+          if (FORCES) {
+            fx += (double)ax;
+            fy += (double)ay;
+            fz += (double)az;
+          }
+        }
+      }
+    }
+    e = (double)pi.w * phi;
+    if (FORCES) {
+      const int64_t o = (int64_t)rec_idx[i] * 3;
+      F[o] = (double)pi.w * fx;
+      F[o + 1] = (double)pi.w * fy;
+      F[o + 2] = (double)pi.w * fz;
+    }
+  }
+  block_partial(e, partial);
+}
 
 // erfc(x) e^(x^2) for x >= 0 as t P(t), t = 1 / (1 + 0.42 x): P is the
 // least relative error polynomial of degree 7 over x in [0, 6.5] (Chebyshev
@@ -368,25 +462,38 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
   *energy = 0.0;
   if (n == 0) return NFFT_OK;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // columns of edge L / ncol >= rcut / kRsReach (at least 9 per side, so the
-  // 7 x 7 around one are distinct), z bins a quarter of that; L / rcut < 3: all pairs
-  const bool cells_form = std::floor(L / rcut) >= 3;
-  const int ncol = cells_form ? std::min((int)std::floor(kRsReach * L / rcut), 128) : 1, nz = 4 * ncol;
-  if (!cells_form && n > 65536) return NFFT_ERR_UNSUPPORTED;   // the all-pairs form is O(n^2)
+  // L / rcut < 3: all pairs
+  const bool sorted = std::floor(L / rcut) >= 3;
+  if (!sorted && n > 65536) return NFFT_ERR_UNSUPPORTED;   // the all-pairs form is O(n^2)
   const int ni = (int)n;
   const int blocks = (ni + kRsThreads - 1) / kRsThreads;
+  int device = 0, sms = 0;
+  if (cudaGetDevice(&device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    cudaGetLastError();
+    return NFFT_ERR_CUDA;
+  }
+  const double partners = 4.0 / 3.0 * M_PI * rcut * rcut * rcut / (L * L * L) * (double)n;
+  const bool cells_form = sorted && partners < cell_partners((double)n / sms);
+  // columns of edge L / side >= rcut / kRsReach (at least 9 per side, so the
+  // 7 x 7 around one are distinct), z bins a quarter of that; or cells of edge
+  // L / side >= rcut / kRsCellReach (at least 6 per side)
+  const int side = !sorted ? 1
+                   : cells_form ? (int)std::min(std::floor(kRsCellReach * L / rcut), 256.0)
+                                : (int)std::min(std::floor(kRsReach * L / rcut), 128.0);
+  const int nz = cells_form ? side : 4 * side;
   // As many ions per warp as still give the chip's resident warps (32 on each
   // of 152 SMs) one each; a warp's ranges serve all its ions in turn.  With 8
   // each throughout, few ions left SMs idle: forces of 2592 ions 395 -> 325 us,
   // 6144: 402 -> 350, 12000: 512 -> 421, 20736: 611 -> 541; 49152: 1155 either way.
   const int per_warp = std::min(std::max(2 * (ni / (2 * 32 * 152)), 2), kRsIons);
   const int per_block = kRsThreads / 32 * per_warp;
-  const int parts = cells_form ? (ni + per_block - 1) / per_block : blocks;
-  const int cells = ncol * ncol * nz;
-  // scratch: partials and the total, and for the cell list records, charges,
+  const int parts = sorted && !cells_form ? (ni + per_block - 1) / per_block : blocks;
+  const int cells = side * side * nz;
+  // scratch: partials and the total, and for the sorted forms records, charges,
   // (cell, rank), columns, counts, starts, scan scratch and record indices
   size_t bytes = sizeof(double) * (size_t)(parts + 1);
-  if (cells_form) {
+  if (sorted) {
     bytes += 16 + (sizeof(float4) + sizeof(int2) + sizeof(float) + sizeof(int)) * ((size_t)n + 1) +
              sizeof(int) * ((size_t)(2 * cells + 2) + (size_t)scan_partials_needed(cells + 1)) +
              (F_dev ? sizeof(int) * (size_t)n : 0);
@@ -402,7 +509,7 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
   };
   double* partial = reinterpret_cast<double*>(buf);
   double* total = partial + parts;
-  if (cells_form) {
+  if (sorted) {
     char* p = buf + sizeof(double) * (size_t)(parts + 1);
     float4* rec = reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(p) + 15) & ~(uintptr_t)15);
     int2* cell_rank = reinterpret_cast<int2*>(rec + n);
@@ -413,29 +520,43 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
     int* scan_scratch = start + cells + 1;
     int* rec_idx = F_dev ? scan_scratch + scan_partials_needed(cells + 1) : nullptr;
     ck(cudaMemsetAsync(count, 0, sizeof(int) * (size_t)(cells + 1), st));
-    k_rs_count<<<blocks, kRsThreads, 0, st>>>(n, r_dev, L, ncol, nz, count, cell_rank);
+    k_rs_count<<<blocks, kRsThreads, 0, st>>>(n, r_dev, L, side, nz, count, cell_rank);
     ck(cudaGetLastError());
     ck(launch_scan(count, start, cells + 1, nullptr, scan_scratch, false, st));   // start[cells] = n
-    k_rs_scatter<<<blocks, kRsThreads, 0, st>>>(n, r_dev, q_dev, L, ncol, nz, start, cell_rank, rec, rec_q, rec_col,
-                                                rec_idx);
-    ck(cudaGetLastError());
-    RsParams P;
-    P.n = ni;
-    P.ncol = ncol;
-    P.nz = nz;
-    P.per_warp = per_warp;
-    P.rc2 = (float)(rcut / L * (rcut / L));
-    P.near = (float)(0.25 * rcut / L);
-    P.alpha = (float)(alpha * L);
-    P.escale = (float)(-alpha * L * alpha * L * 1.4426950408889634);
-    P.c2 = (float)(kTwoOverSqrtPi * alpha * L);
-    P.phi_scale = 1.0 / L;
-    P.f_scale = 1.0 / (L * L);
-    if (F_dev)
-      k_rs_columns<true><<<parts, kRsThreads, 0, st>>>(P, rec, rec_q, rec_col, start, partial, rec_idx, F_dev);
-    else
-      k_rs_columns<false><<<parts, kRsThreads, 0, st>>>(P, rec, rec_q, rec_col, start, partial, nullptr, nullptr);
-    ck(cudaGetLastError());
+    if (cells_form) {
+      k_rs_scatter_cells<<<blocks, kRsThreads, 0, st>>>(n, r_dev, q_dev, L, side, start, cell_rank, rec, rec_col,
+                                                        rec_idx);
+      ck(cudaGetLastError());
+      const float h = (float)(L / side), rc2 = (float)(rcut * rcut);
+      if (F_dev)
+        k_rs_cells<true><<<blocks, kRsThreads, 0, st>>>(ni, side, h, rc2, (float)alpha, rec, rec_col, start, partial,
+                                                        rec_idx, F_dev);
+      else
+        k_rs_cells<false><<<blocks, kRsThreads, 0, st>>>(ni, side, h, rc2, (float)alpha, rec, rec_col, start, partial,
+                                                         nullptr, nullptr);
+      ck(cudaGetLastError());
+    } else {
+      k_rs_scatter<<<blocks, kRsThreads, 0, st>>>(n, r_dev, q_dev, L, side, nz, start, cell_rank, rec, rec_q, rec_col,
+                                                  rec_idx);
+      ck(cudaGetLastError());
+      RsParams P;
+      P.n = ni;
+      P.ncol = side;
+      P.nz = nz;
+      P.per_warp = per_warp;
+      P.rc2 = (float)(rcut / L * (rcut / L));
+      P.near = (float)(0.25 * rcut / L);
+      P.alpha = (float)(alpha * L);
+      P.escale = (float)(-alpha * L * alpha * L * 1.4426950408889634);
+      P.c2 = (float)(kTwoOverSqrtPi * alpha * L);
+      P.phi_scale = 1.0 / L;
+      P.f_scale = 1.0 / (L * L);
+      if (F_dev)
+        k_rs_columns<true><<<parts, kRsThreads, 0, st>>>(P, rec, rec_q, rec_col, start, partial, rec_idx, F_dev);
+      else
+        k_rs_columns<false><<<parts, kRsThreads, 0, st>>>(P, rec, rec_q, rec_col, start, partial, nullptr, nullptr);
+      ck(cudaGetLastError());
+    }
   } else {
     if (F_dev)
       k_rs_pairs<true><<<blocks, kRsThreads, 0, st>>>(ni, r_dev, q_dev, L, rcut, alpha, partial, F_dev);
