@@ -3,8 +3,8 @@
 // over the pairs (and periodic images) closer than a cut-off r_c; the primed
 // sum omits n = 0 for i = j.
 //
-// Two forms, chosen by the box:
-//   - cell list (L / r_c >= 3): the box is cut into columns along z of edge
+// Three forms:
+//   - columns (L / r_c >= 3): the box is cut into columns along z of edge
 //     L / ncol >= r_c / 3, each cut into fine z bins, and the ions are
 //     counting-sorted by (column, bin), so a column's ions are contiguous and
 //     nearly ordered by z.  A warp takes two ions of one column; for each of
@@ -14,25 +14,35 @@
 //     47% of the candidates are partners; of the 125 cells of edge r_c / 2
 //     around an ion, a thread per ion, 23% were, and every candidate ran the
 //     whole pair term because one lane of 32 accepted it.  393216 ions,
-//     r_c = 10, about 4000 partners each, with forces: 12.8 -> 4.7 ms.  It is
-//     bound by issue (70 instructions per 64 candidates, 60% of the slots) and
-//     the FP32 pipe (25 of them paired operations of two cycles).
-//     With r_c <= L / 3 only the minimum image of a pair can be within r_c,
-//     and it is found exactly once.  Lengths are in units of L.  An ion's x
-//     and y are FP32 offsets from its column's axis, its z the sum of a
-//     multiple of 2^-10 and an FP32 remainder, so that separations carry an
-//     error of about 1e-9 L and neither box coordinates nor periodic shifts
-//     are rounded; pair terms and the sums over a range are FP32, an ion's sums
+//     r_c = 10, about 4000 partners each, with forces, a call: 13.2 -> 5.5 ms
+//     (5.2 with FP32 sums per ion).  It is bound by issue and the FP32 pipe: 70
+//     instructions per 64 candidates, 25 of them paired operations of two cycles,
+//     and about 35 per range for its sums;
+//     Lengths are in units of L.  An ion's x and y are FP32 offsets from its
+//     column's axis, its z the sum of a multiple of 2^-10 and an FP32 remainder:
+//     a separation along z is rounded to FP32 once, along x and y with its
+//     columns' distance and its offsets, an error of at most 2e-8 L between
+//     neighbours and 5e-8 L between third neighbours of 9 columns a side, 1.2e-9 and
+//     2e-9 L of 128.  Pair terms and the sums over a range are FP32, an ion's sums
 //     over its ranges FP64;
+//   - the same with few partners and many ions (cell_partners): cells of edge
+//     L / nc >= r_c / 2, a thread per ion over the 5^3 cells around its own.  A
+//     range of the columns then holds fewer ions than a warp has lanes (13 of 32
+//     at 250 partners), while this form's work falls with the partners.  FP32
+//     offsets from the cells' centres, FP32 pair terms and sums over a cell, FP64
+//     over the cells;
+//     In both, with r_c <= L / 3 only the minimum image of a pair can be within
+//     r_c, and it is found exactly once;
 //   - all pairs (smaller boxes): the minimum image of every pair plus the 26
 //     shifts by L, all in FP64, which is the definition itself (r_c < L).
-// The energy 1/2 sum_i q_i phi_i is reduced in FP64 in a fixed order (block
-// partials, then one block over the partials), so it is the same run to run.
+// The energy 1/2 sum_i q_i phi_i is reduced in FP64, the blocks' partials in a
+// fixed order; the order of ions inside a bin (atomics) and with it the last
+// bits of an ion's FP32 sums change from run to run.
 //
 // Forces (the negative gradient of Eq. 11; the paper names MD as the use but
 // prints no force formula): F_i = q_i sum_j q_j g(d) (r_i - r_j + n L) with
 // g(d) = (erfc(alpha d) / d + 2 alpha / sqrt(pi) exp(-alpha^2 d^2)) / d^2,
-// summed by the same two forms (each ion sums its own force, no atomics).
+// summed by the same forms (each ion sums its own force, no atomics).
 #include <cmath>
 #include <cstdint>
 
