@@ -493,10 +493,10 @@ int real_space_impl(int64_t n, const double* r_dev, const double* q_dev, double 
                                 : (int)std::min(std::floor(kRsReach * L / rcut), 128.0);
   const int nz = cells_form ? side : 4 * side;
   // As many ions per warp as still give the chip's resident warps (32 on each
-  // of 152 SMs) one each; a warp's ranges serve all its ions in turn.  With 8
+  // SM) one each; a warp's ranges serve all its ions in turn.  With 8
   // each throughout, few ions left SMs idle: forces of 2592 ions 395 -> 325 us,
   // 6144: 402 -> 350, 12000: 512 -> 421, 20736: 611 -> 541; 49152: 1155 either way.
-  const int per_warp = std::min(std::max(2 * (ni / (2 * 32 * 152)), 2), kRsIons);
+  const int per_warp = std::min(std::max(2 * (ni / (2 * 32 * sms)), 2), kRsIons);
   const int per_block = kRsThreads / 32 * per_warp;
   const int parts = sorted && !cells_form ? (ni + per_block - 1) / per_block : blocks;
   const int cells = side * side * nz;
