@@ -188,7 +188,7 @@ typedef struct {
   int threads;               /* threads per block of the point kernels */
   int64_t device_bytes;      /* device memory held by the plan (grids, sort buffers, tables) */
   double sigma[3];           /* actual n_t / N_t */
-  int max_subproblem;        /* points per subproblem in use */
+  int max_subproblem;        /* points per subproblem in use: at most; a bin's pieces are even */
   int spread_threads;        /* NFFT_OPT_SPREAD_THREADS (0 = chosen per launch) */
   int interp_threads;        /* NFFT_OPT_INTERP_THREADS (0 = chosen per launch) */
   int sparse_points;         /* spreading subproblems below this many points use the grid-warp kernel */

@@ -423,6 +423,17 @@ __global__ void k_sub_count(SortArgs s, const int* __restrict__ key_start, int P
   sub_count[b] = (cnt + P - 1) / P;
 }
 
+// Points of a bin's pieces: at most P, and as even as can be (pencils: P, whole
+// batches of their kernels).  In pieces of P and the rest, uniform points make
+// tiles for a few points each: 2-D, N = 256^2, 100,000 points, bins of 390, P =
+// 328, spreading + interpolation at 12 taps: FP32 149 + 74 us, even 118 + 45,
+// three right-hand sides 347 + 227, even 280 + 149; FP64 447 + 430, even 320 + 266.
+__device__ __forceinline__ int piece_size(int count, int P, int fine) {
+  if (fine > 1) return P;
+  const int pieces = max((count + P - 1) / P, 1);
+  return (count + pieces - 1) / pieces;
+}
+
 __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const int* __restrict__ bin_start,
                            const int* __restrict__ sub_start, int P, SubProblem* __restrict__ subs) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -432,11 +443,12 @@ __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const 
   const int item = find_item<int>(s.bin_offsets, s.n_items, b);
   const int local_bin = b - s.bin_offsets[item];
   const int s0 = sub_start[b];
-  for (int k = 0, off = 0; off < cnt; ++k, off += P) {
+  const int size = piece_size(cnt, P, s.items[item].geom.fine);
+  for (int k = 0, off = 0; off < cnt; ++k, off += size) {
     SubProblem sp;
     sp.bin = local_bin;
     sp.start = bin_start[b] + off;
-    sp.count = min(P, cnt - off);
+    sp.count = min(size, cnt - off);
     sp.item = item;
     sp.dense = 0;
     subs[s0 + k] = sp;
@@ -488,11 +500,12 @@ __global__ void __launch_bounds__(1024) k_subproblems(SortArgs s, const int* __r
   for (int t = threadIdx.x; t < total; t += 1024) {
     const int b = find_item<int>(sub_start, nb, t);   // the last bin that starts at t or before: not an empty one
     const int item = find_item<int>(s.bin_offsets, s.n_items, b);
-    const int off = (t - sub_start[b]) * P;
+    const int size = piece_size(bin_count[b], P, s.items[item].geom.fine);
+    const int off = (t - sub_start[b]) * size;
     SubProblem sp;
     sp.bin = b - s.bin_offsets[item];
     sp.start = bin_start[b] + off;
-    sp.count = min(P, bin_count[b] - off);
+    sp.count = min(size, bin_count[b] - off);
     sp.item = item;
     sp.dense = 0;
     subs[t] = sp;
