@@ -183,8 +183,9 @@ __global__ void __launch_bounds__(256) k_spread_wpp(PointKernelArgs<Real> a, Wpp
   }
 }
 
+// five blocks of 256 threads per SM in FP32 (at most 48 registers), four in FP64 (64)
 template <int D, int W, typename Real>
-__global__ void __launch_bounds__(256) k_interp_wpp(PointKernelArgs<Real> a, WppLayout lay) {
+__global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 5 : 4) k_interp_wpp(PointKernelArgs<Real> a, WppLayout lay) {
   using C = typename Cplx<Real>::type;
   using S = WppShape<D, W>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
