@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(PencilShape<W, NR>::THREADS, PencilShape<W, NR
 //     so for the others.
 template <int W, int NR>
 struct SlabShape {
-  static constexpr int THREADS = W <= 6 ? 192 : NR == 2 || W >= 14 ? 128 : 256;
+  static constexpr int THREADS = W <= 6 ? 192 : W <= 12 ? 128 : 256;
   static constexpr int SIDE = 8 * NR;   // tile columns per dimension
   // pitch of a tile row in cells, and whether a lane's rows are neighbours
   // (row q PASSES + k) or Q apart (q + Q k): the fewest wavefronts over all
@@ -379,10 +379,17 @@ struct SlabShape {
   static constexpr int PITCH = W == 2 ? 18 : W == 4 ? 20 : W == 6 ? 22 : W == 8 ? 20 : W <= 12 ? 26 : W == 14 ? 30 : 24;
   static constexpr bool NEIGHBOURS = W == 8 || W == 12;
   static constexpr int PLANE = SIDE * PITCH;
-  // (8 taps, uniform, M = 10^6: 254 us for 3 planes, 236 for 4, 213 for 7, 206
-  // for 9, 210 for 12; 96000 points, three right-hand sides: 346, 259, 219,
-  // 195, 180.  More planes mean fewer reloads and fewer resident blocks)
-  static constexpr int AHEAD = W == 8 ? 9 : NR == 2 ? 7 : W == 12 ? 2 : 1;   // planes of points a slab serves
+  // (a slab is loaded whole, AHEAD + W - 1 planes, for every AHEAD planes of
+  // points: more planes mean fewer reloads and fewer resident blocks.  8 taps,
+  // uniform, M = 10^6: 254 us for 3 planes, 236 for 4, 213 for 7, 206 for 9, 210
+  // for 12; 96000 points, three right-hand sides: 346, 259, 219, 195, 180.
+  // N = 96^3, one right-hand side, 2 / 8 points per plane: 6 taps 105 / 151 us
+  // for 7 planes, 86 / 131 for 12; 12 taps 459 / 634 for 2 planes and 256 threads,
+  // 206 / 401 for 7 and 128, 217 / 428 for 12 and 256; 14 taps 1077 / 1627 for 1
+  // and 128, 538 / 854 for 4 and 256, 321 / 623 for 12 and 256; 16 taps 1791 / 2628
+  // for 1 and 128, 588 / 1126 for 8 and 256, 475 / 1006 for 14 and 256; 10 taps
+  // 289 / 583 for 7, 264 / 564 for 12)
+  static constexpr int AHEAD = W == 6 || W == 14 ? 12 : W == 8 ? 9 : W == 16 ? 14 : 7;   // planes of points a slab serves
   static constexpr int PLANES = AHEAD + W - 1;
   static constexpr int Q = 32 / W, PASSES = (W + Q - 1) / Q;
   static constexpr bool FULL = 32 % W == 0 && Q * PASSES == W;
