@@ -242,8 +242,11 @@ struct SubProblem {
   int start;   // first sorted position
   int count;
   int item;
-  int dense;   // pencils: points share cells (kDenseRun of them per cell or more)
+  int form;    // how its points are interpolated (pencils)
 };
+constexpr int kFormGrid = 0;    // few points per plane: a warp per point straight from the grid
+constexpr int kFormSlab = 1;    // a warp per point from a slab of planes
+constexpr int kFormDense = 2;   // points share cells (kDenseRun of them per cell or more): a thread per point from a slab
 
 struct GridGeom {
   int d;
@@ -287,6 +290,7 @@ struct SortedPoints {
   const int* sub_start;      // exclusive scan of subproblems per global bin
   const int* num_subs;       // device scalar: all subproblems
   const int* bin_count;      // points per global bin
+  const int* grid_points;   // per item: points of its kFormGrid subproblems (pencils)
   const int* bin_start;      // first sorted position per global bin
 };
 

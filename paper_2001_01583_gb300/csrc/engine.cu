@@ -427,6 +427,7 @@ int Engine::release_layout() {
   free_dev(sub_start);
   free_dev(scan_partials);
   free_dev(num_subs);
+  free_dev(grid_points);
   free_dev(subs);
   free_dev(key_rank);
   free_dev(perm);
@@ -581,11 +582,14 @@ int Engine::build_layout() {
     // pencils (points_pencil.cuh): 3-D items in FP32 with nothing chosen by
     // the caller that belongs to the other kernels (method, bins, split, owner
     // or tensor-core form), and at least a point per plane of a pencil on
-    // average.  Below that the window moves on with every point and is written
-    // out for it alone, as the grid-warp kernels do without sorting by plane:
-    // N = 64^3, 8 taps, one set: 20,000 points (0.8 per plane) take 174 us in
-    // pencils and 166 us on the other kernels, 96,000 points (3.7) 19 us
-    // against 36 to spread and 72 against 103 to interpolate one right-hand side.
+    // average.  Below that the window moves on with every point
+    // and is written out for it alone, as the grid-warp kernels do without
+    // sorting by plane.  Spreading uniform points on N = 64^3 and 96^3, the
+    // other kernels' time over the pencils' at 1 / 2 / 4 points per plane:
+    // 2 taps 0.9 / 1.2 / 1.25 and 1.4 / 1.4 / 1.6, 4 taps 1.0 / 1.4 / 1.4 and
+    // 1.2 / 1.2 / 1.5, 6 taps 1.1 / 1.7 / 3.7 and 1.1 / 1.5 / 4.3, 8 taps
+    // 1.6 / 2.2 / 1.9 and 1.6 / 2.8 / 2.3, 12 taps 2.7 / 5.3 / 3.9 and 2.5 / 6.3 /
+    // 5.4; the sort takes up to 8 us more with the planes' keys.
     const PencilLaunch pl = pencil_launch_f32(c.taps, true);
     c.pencil = s.d == 3 && method_opt == NFFT_METHOD_AUTO && method == NFFT_METHOD_WARP &&
                precision == NFFT_FP32_MIXED && !explicit_bins && sparse_opt == 0 && sparse_interp_opt == 0 &&
@@ -747,6 +751,7 @@ int Engine::build_layout() {
       kc.sparse_points_interp = c.sparse_interp;
       kc.owner = c.owner;
       kc.pencil = c.pencil;
+      kc.pencil_split = false;
       kc.tensor = c.tensor;
       kc.tensor_interp = c.tensor_interp;
       kc.item_begin = k;
@@ -760,6 +765,16 @@ int Engine::build_layout() {
     kc.bin_end = bin_off[k + 1];
     kc.max_nrhs = std::max(kc.max_nrhs, it.nrhs);
     kc.max_subs += nb_total + s.M / max_sub + 1;
+  }
+  for (auto& kc : kclasses) {   // pencils below the slabs' points per plane on average
+    if (!kc.pencil) continue;
+    const PencilLaunch l = pencil_launch_f32(kc.taps, false);
+    double points = 0.0, cells = 0.0;
+    for (int k = kc.item_begin; k < kc.item_end; ++k) {
+      points += (double)items[k].M;
+      cells += (double)items[k].geom.grid_cells;
+    }
+    kc.pencil_split = 2.0 * points * l.edge * l.edge < l.slab_points * cells;
   }
   total_points = pts_off[nitems];
   if (total_points > (int64_t)INT32_MAX) return NFFT_ERR_UNSUPPORTED;   // 32-bit sort indices
@@ -787,6 +802,7 @@ int Engine::build_layout() {
   TRY(alloc_dev(sub_start, sizeof(int) * B, device_bytes));
   TRY(alloc_dev(scan_partials, sizeof(int) * (size_t)scan_partials_needed((int)std::max(B, K)), device_bytes));
   TRY(alloc_dev(num_subs, sizeof(int), device_bytes));
+  TRY(alloc_dev(grid_points, sizeof(int) * nitems, device_bytes));
   TRY(alloc_dev(subs, sizeof(SubProblem) * (size_t)max_subs_total, device_bytes));
   TRY(alloc_dev(key_rank, sizeof(int2) * P, device_bytes));
   TRY(alloc_dev(perm, sizeof(int) * P, device_bytes));
@@ -1035,6 +1051,7 @@ int Engine::run_points(const KClass& kc, bool spread, const void* in, void* out,
   a.pts.num_subs = num_subs;
   a.pts.bin_count = bin_count;
   a.pts.bin_start = bin_start;
+  a.pts.grid_points = grid_points;
   a.items = table ? table : d_items;
   a.item_begin = kc.item_begin;
   a.item_end = kc.item_end;
@@ -1047,9 +1064,15 @@ int Engine::run_points(const KClass& kc, bool spread, const void* in, void* out,
   const int max_nrhs = in ? nrhs : kc.max_nrhs;
   a.sub_min_count = 0;
   a.sub_max_count = INT_MAX;
+  a.gm_split_log2 = kGmSplitLog2;
   a.err = err_flag;
   if constexpr (sizeof(Real) == 4)
-    if (kc.pencil) return run_pencil(kc, a, spread, max_nrhs);
+    if (kc.pencil) {
+      a.split_forms = !spread && kc.pencil_split;
+      TRY(run_pencil(kc, a, spread, max_nrhs));
+      if (!a.split_forms) return NFFT_OK;
+      return run_gm<Real>(kc, a, false);
+    }
   if (kc.method == NFFT_METHOD_GRID_WARP) return run_gm<Real>(kc, a, spread);
   if (kc.method == NFFT_METHOD_GLOBAL) return run_global<Real>(kc, a, spread);
   // tiled kernels take the bins of at least `split` points, the owner
@@ -1104,7 +1127,7 @@ int Engine::run_owner(const KClass& kc, PointKernelArgs<Real>& a) {
   return NFFT_OK;
 }
 
-// One warp per point straight on the grid; kGmSplitHost warps share a subproblem.
+// One warp per point straight on the grid; 2^a.gm_split_log2 warps share a subproblem.
 template <typename Real>
 int Engine::run_gm(const KClass& kc, PointKernelArgs<Real>& a, bool spread) {
   const void* fn = precision == NFFT_FP64 ? gm_kernel_f64(kc.d, kc.taps, spread) : gm_kernel_f32(kc.d, kc.taps, spread);
@@ -1113,7 +1136,11 @@ int Engine::run_gm(const KClass& kc, PointKernelArgs<Real>& a, bool spread) {
   const int threads = 32 * kGmWarpsHost;
   const int per_sm = std::max(1, blocks_per_sm(fn, threads, 0));
   int64_t blocks = (int64_t)per_sm * num_sms;
-  const int64_t need = (kc.max_subs * kGmSplitHost + kGmWarpsHost - 1) / kGmWarpsHost;
+  // a pencil's subproblems hold 32 points and more: up to 16 warps each while all fit the chip
+  if (kc.pencil)
+    while (a.gm_split_log2 < kGmSplitLog2Pencil && (kc.max_subs << (a.gm_split_log2 + 1)) <= blocks * kGmWarpsHost)
+      ++a.gm_split_log2;
+  const int64_t need = ((kc.max_subs << a.gm_split_log2) + kGmWarpsHost - 1) / kGmWarpsHost;
   if (blocks > need) blocks = need;
   if (blocks < 1) blocks = 1;
   void* args[] = {&a};
@@ -1336,12 +1363,12 @@ int Engine::set_points_impl(const double* x_override) {
   Real* d[3] = {static_cast<Real*>(delta[0]), static_cast<Real*>(delta[1]), static_cast<Real*>(delta[2])};
   CK(launch_scatter<Real>(s, key_start, key_rank, perm, local, d, stream));
   CK(launch_subproblems(s, key_start, max_sub, bin_count, bin_start, sub_count, sub_start, num_subs, scan_partials,
-                        subs, stream));
+                        subs, grid_points, stream));
   if constexpr (sizeof(Real) == 4) {
     bool pencils = false;
     for (const auto& kc : kclasses) pencils = pencils || kc.pencil;
     if (pencils && s.total_points > 0) {
-      CK(launch_refine(s, max_subs_total, subs, num_subs, perm, local, d, stream));
+      CK(launch_refine(s, max_subs_total, subs, num_subs, perm, local, d, grid_points, stream));
       ++kernel_launches;
     }
   }

@@ -42,6 +42,7 @@ struct KClass {
   int sparse_points;          // spreading subproblems below this many points: grid-warp kernel (0: none)
   int sparse_points_interp;   // the same for interpolation
   bool pencil;                // 3-D FP32 pencils (points_pencil.cuh)
+  bool pencil_split;          // and few points per plane: interpolation by the subproblems' forms, two launches
   bool owner;                 // spreading of sparse bins by the owner kernel (3-D)
   bool tensor;                // dense bins spread on the tensor cores (3-D, FP32)
   bool tensor_interp;         // dense bins interpolated on the tensor cores (3-D, FP32)
@@ -211,6 +212,7 @@ class Engine {
   int* scan_partials = nullptr;   // scratch of the multi-block scans
   int* sub_start = nullptr;
   int* num_subs = nullptr;
+  int* grid_points = nullptr;     // per item: points of its kFormGrid subproblems (pencils)
   SubProblem* subs = nullptr;
   int2* key_rank = nullptr;
   int* perm = nullptr;

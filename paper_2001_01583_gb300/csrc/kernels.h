@@ -46,11 +46,13 @@ cudaError_t launch_scatter(const SortArgs& s, const int* key_start, const int2* 
 int subproblem_launches(int nbins);
 cudaError_t launch_subproblems(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
                                int* sub_count, int* sub_start, int* num_subs, int* partials, SubProblem* subs,
-                               cudaStream_t st);
+                               int* grid_points, cudaStream_t st);
 // Pencil items (GridGeom::fine > 1): the points of every subproblem ordered by
 // cell and their records written (the scatter writes their indices only).
+// grid_points: per item, the points of its kFormGrid subproblems
+// (launch_subproblems clears it).
 cudaError_t launch_refine(const SortArgs& s, int64_t max_subs, SubProblem* subs, const int* num_subs, int* perm,
-                          uint32_t* local, float* const* delta, cudaStream_t st);
+                          uint32_t* local, float* const* delta, int* grid_points, cudaStream_t st);
 
 // ---- spreading / interpolation ---------------------------------------------
 template <typename Real>
@@ -66,6 +68,8 @@ struct PointKernelArgs {
   int nrhs;
   // subproblems whose bin holds sub_min_count <= points < sub_max_count are this launch's
   int sub_min_count, sub_max_count;
+  int split_forms;            // pencils: interpolation by slab_takes
+  int gm_split_log2;          // warps that share a subproblem (grid-warp kernels)
   int item_begin, item_end;   // the launch's items (internal order)
   int* err;                   // device error flag: kernels that give up a wait set bit 1
 };
@@ -75,6 +79,15 @@ template <typename Real>
 __device__ __forceinline__ bool sub_selected(const PointKernelArgs<Real>& a, const SubProblem& s) {
   const int total = a.pts.bin_count[a.items[s.item].bin_offset + s.bin];
   return total >= a.sub_min_count && total < a.sub_max_count;
+}
+
+// Pencils of few points: the slab kernel interpolates a subproblem, or the
+// grid-warp kernel, which takes an item's (but the dense ones) where those of
+// few points per plane hold most of its points: work for both launches, one
+// after the other, cost more than the better form of either saved.
+template <typename Real>
+__device__ __forceinline__ bool slab_takes(const PointKernelArgs<Real>& a, const SubProblem& s) {
+  return s.form == kFormDense || 2 * (int64_t)a.pts.grid_points[s.item] <= a.items[s.item].M;
 }
 
 // The launch's subproblems: [lo, hi).
@@ -111,7 +124,8 @@ const void* global_kernel_f64(bool spread);
 // Warp-per-point kernels straight on the grid (points_gm.cuh), any d, taps 2..26 even;
 // blocks of kGmWarpsHost warps.
 constexpr int kGmWarpsHost = 8;
-constexpr int kGmSplitHost = 4;   // warps sharing one subproblem
+constexpr int kGmSplitLog2 = 2;         // 4 warps share a subproblem (usually a bin of few points),
+constexpr int kGmSplitLog2Pencil = 4;   // up to 16 a pencil's, where they all fit the chip
 const void* gm_kernel_f32(int d, int taps, bool spread);
 const void* gm_kernel_f64(int d, int taps, bool spread);
 
@@ -147,8 +161,25 @@ struct PencilLaunch {
   int threads;
   size_t smem;
   int edge;
+  int slab_points;   // points per plane (times two) from which a slab is worth loading
 };
 PencilLaunch pencil_launch_f32(int taps, bool spread);
+// Planes of points a slab serves.
+__host__ __device__ constexpr int slab_ahead(int taps) {
+  return taps == 6 || taps == 14 ? 12 : taps == 8 ? 9 : taps == 16 ? 14 : 7;
+}
+// Points per plane of a pencil (times two) from which interpolation loads slabs
+// of its planes; below, the grid-warp kernel reads the cells of each point
+// alone (W^3 of them; a slab is up to 24^2 cells per plane).  Where the two
+// meet.  Grid-warp / slabs, uniform points, N = 96^3, one right-hand side, us at
+// 1, 2, 4, 8 points per plane: 4 taps 26/42, 45/47, 69/53, 126/61; 6 taps 49/75,
+// 84/86, 150/102, 265/131; 8 taps 67/117, 121/131, 221/158, 434/214; 10 taps
+// 226/238, 433/289, 838/391; 12 taps 88/167, 162/206, 281/275, 524/401; 14 taps
+// 170/272, 326/321, 644/414; 16 taps 243/374, 471/475, 860/658.  (N = 64^3 and
+// three right-hand sides meet a little higher for 4, 12 and 16 taps.)
+__host__ __device__ constexpr int slab_points(int taps) {
+  return taps <= 4 ? 6 : taps == 6 ? 4 : taps == 8 ? 5 : taps == 10 ? 2 : taps == 12 ? 10 : taps == 14 ? 4 : 6;
+}
 constexpr int kDenseRun = 4;   // points per occupied cell from which a pencil's subproblem is dense
 
 // 3-D spreading on the tensor cores (points_tc.cuh): FP32, taps 4, 6 or 8,

@@ -11,6 +11,7 @@ PencilLaunch pencil_launch_f32(int taps, bool spread) {
                   : reinterpret_cast<const void*>(&k_interp_pencil<W, NR>);                                \
     l.threads = spread ? PencilShape<W, NR>::THREADS : SlabShape<W, NR>::THREADS;                          \
     l.smem = spread ? pencil_smem_bytes<W, NR>() : SlabShape<W, NR>::smem_bytes();                         \
+    l.slab_points = slab_points(W);                                                                        \
     l.edge = 8 * NR + 1 - W;                                                                               \
   }
   GBNFFT_PENCIL_CASES(GBNFFT_PENCIL)

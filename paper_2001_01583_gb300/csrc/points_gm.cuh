@@ -4,8 +4,8 @@
 //
 // A shared tile pays for zeroing, loading and flushing (b + W - 1)^d cells
 // per subproblem; with a few points per bin that costs more than the points'
-// own W^d cell updates.  Here kGmSplit warps share a subproblem, each taking
-// every kGmSplit-th point, with no tile and no block barrier:
+// own W^d cell updates.  Here 4 (16) warps share a subproblem, each taking
+// every fourth (16th) point, with no tile and no block barrier:
 //   - lanes split the point's d * W window weights into a per-warp table;
 //   - lanes cover one plane of the point's footprint (W x W cells, the last
 //     two dimensions; W cells in 1-D) in ceil(W^2 / 32) passes, lanes along
@@ -29,7 +29,6 @@ struct GmShape {
 };
 
 constexpr int kGmWarps = kGmWarpsHost;   // warps per block
-constexpr int kGmSplit = kGmSplitHost;   // warps sharing one subproblem's points
 // resident blocks asked of the compiler: the kernels wait on global loads,
 // so narrow windows trade registers (at most 64) for more warps
 template <int W>
@@ -92,11 +91,12 @@ __global__ void __launch_bounds__(32 * kGmWarps, gm_min_blocks<W>()) k_spread_gm
   int lo, hi;
   launch_subs(a, lo, hi);
   const int64_t stride = (int64_t)gridDim.x * kGmWarps;
-  const int64_t work = (int64_t)(hi - lo) * kGmSplit;
+  const int split = 1 << a.gm_split_log2;
+  const int64_t work = (int64_t)(hi - lo) << a.gm_split_log2;
   for (int64_t wi = (int64_t)blockIdx.x * kGmWarps + warp; wi < work; wi += stride) {
-    const int sp = lo + (int)(wi / kGmSplit), part = (int)(wi % kGmSplit);
+    const int sp = lo + (int)(wi >> a.gm_split_log2), part = (int)wi & (split - 1);
     const SubProblem sub = a.pts.subs[sp];
-    if (part >= sub.count || !sub_selected(a, sub)) continue;
+    if (part >= sub.count || !sub_selected(a, sub) || (a.split_forms && slab_takes(a, sub))) continue;
     const ItemDev& it = a.items[sub.item];
     const GridGeom& g = it.geom;
     const ItemCall call = item_call(a, it);
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(32 * kGmWarps, gm_min_blocks<W>()) k_spread_gm
     int bc[kMaxDim];
     bin_coords(sub.bin, g, bc);
     const int64_t plane_cells = D == 3 ? (int64_t)g.n[1] * g.n[2] : 0;
-    for (int pp = part; pp < sub.count; pp += kGmSplit) {
+    for (int pp = part; pp < sub.count; pp += split) {
       const int idx = sub.start + pp;
       const int j = a.pts.perm[idx];
       GmPoint<D, W, Real> q;
@@ -146,11 +146,12 @@ __global__ void __launch_bounds__(32 * kGmWarps, gm_min_blocks<W>()) k_interp_gm
   int lo, hi;
   launch_subs(a, lo, hi);
   const int64_t stride = (int64_t)gridDim.x * kGmWarps;
-  const int64_t work = (int64_t)(hi - lo) * kGmSplit;
+  const int split = 1 << a.gm_split_log2;
+  const int64_t work = (int64_t)(hi - lo) << a.gm_split_log2;
   for (int64_t wi = (int64_t)blockIdx.x * kGmWarps + warp; wi < work; wi += stride) {
-    const int sp = lo + (int)(wi / kGmSplit), part = (int)(wi % kGmSplit);
+    const int sp = lo + (int)(wi >> a.gm_split_log2), part = (int)wi & (split - 1);
     const SubProblem sub = a.pts.subs[sp];
-    if (part >= sub.count || !sub_selected(a, sub)) continue;
+    if (part >= sub.count || !sub_selected(a, sub) || (a.split_forms && slab_takes(a, sub))) continue;
     const ItemDev& it = a.items[sub.item];
     const GridGeom& g = it.geom;
     const ItemCall call = item_call(a, it);
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(32 * kGmWarps, gm_min_blocks<W>()) k_interp_gm
     int bc[kMaxDim];
     bin_coords(sub.bin, g, bc);
     const int64_t plane_cells = D == 3 ? (int64_t)g.n[1] * g.n[2] : 0;
-    for (int pp = part; pp < sub.count; pp += kGmSplit) {
+    for (int pp = part; pp < sub.count; pp += split) {
       const int idx = sub.start + pp;
       const int j = a.pts.perm[idx];
       GmPoint<D, W, Real> q;

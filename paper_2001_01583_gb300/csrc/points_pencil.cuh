@@ -389,7 +389,7 @@ struct SlabShape {
   // and 128, 538 / 854 for 4 and 256, 321 / 623 for 12 and 256; 16 taps 1791 / 2628
   // for 1 and 128, 588 / 1126 for 8 and 256, 475 / 1006 for 14 and 256; 10 taps
   // 289 / 583 for 7, 264 / 564 for 12)
-  static constexpr int AHEAD = W == 6 || W == 14 ? 12 : W == 8 ? 9 : W == 16 ? 14 : 7;   // planes of points a slab serves
+  static constexpr int AHEAD = slab_ahead(W);   // planes of points a slab serves
   static constexpr int PLANES = AHEAD + W - 1;
   static constexpr int Q = 32 / W, PASSES = (W + Q - 1) / Q;
   static constexpr bool FULL = 32 % W == 0 && Q * PASSES == W;
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(SlabShape<W, NR>::THREADS) k_interp_pencil(Poi
   int* jt = off + T;
   int* col = jt + T;                                                   // grid index of a tile column in its plane
   SubProblem sub;
-  if (!pencil_sub(a, sub)) return;
+  if (!pencil_sub(a, sub) || (a.split_forms && !slab_takes(a, sub))) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const ItemDev& it = a.items[sub.item];
   const GridGeom& g = it.geom;
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(SlabShape<W, NR>::THREADS) k_interp_pencil(Poi
       }
     }
     const int cell = (l0 - base) * S::PLANE + unpack_local(loc, 3, 1) * S::PITCH + unpack_local(loc, 3, 2);
-    if (sub.dense) {
+    if (sub.form == kFormDense) {
       float wy[W], wx[W];
       if (mine) {
         window_taps<W>(win, 0, d0, wx);

@@ -435,8 +435,10 @@ __device__ __forceinline__ int piece_size(int count, int P, int fine) {
 }
 
 __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const int* __restrict__ bin_start,
-                           const int* __restrict__ sub_start, int P, SubProblem* __restrict__ subs) {
+                           const int* __restrict__ sub_start, int P, SubProblem* __restrict__ subs,
+                           int* __restrict__ grid_points) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < s.n_items) grid_points[b] = 0;   // (an item has a bin or more)
   if (b >= s.total_bins) return;
   const int cnt = bin_count[b];
   if (cnt == 0) return;
@@ -450,7 +452,7 @@ __global__ void k_sub_fill(SortArgs s, const int* __restrict__ bin_count, const 
     sp.start = bin_start[b] + off;
     sp.count = min(size, cnt - off);
     sp.item = item;
-    sp.dense = 0;
+    sp.form = kFormGrid;
     subs[s0 + k] = sp;
   }
 }
@@ -463,7 +465,8 @@ constexpr int kSubSingle = 16384;
 __global__ void __launch_bounds__(1024) k_subproblems(SortArgs s, const int* __restrict__ key_start, int P,
                                                        int* __restrict__ bin_count, int* __restrict__ bin_start,
                                                        int* __restrict__ sub_start, int* __restrict__ num_subs,
-                                                       SubProblem* __restrict__ subs) {
+                                                       SubProblem* __restrict__ subs, int* __restrict__ grid_points) {
+  for (int i = threadIdx.x; i < s.n_items; i += 1024) grid_points[i] = 0;
   __shared__ int wsum[32];
   const int nb = s.total_bins, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int chunk = (nb + 1023) / 1024;
@@ -507,7 +510,7 @@ __global__ void __launch_bounds__(1024) k_subproblems(SortArgs s, const int* __r
     sp.start = bin_start[b] + off;
     sp.count = min(size, bin_count[b] - off);
     sp.item = item;
-    sp.dense = 0;
+    sp.form = kFormGrid;
     subs[t] = sp;
   }
 }
@@ -516,7 +519,7 @@ __global__ void __launch_bounds__(1024) k_subproblems(SortArgs s, const int* __r
 // planes, by their indices only): their records written, in runs of kRefine
 // points, ordered by cell, (l0, l1, l2), where there are as many points as
 // cells.  Neighbouring points then share cells, which interpolation turns into
-// shared-memory broadcasts (SubProblem::dense).  The scatter writes 4 bytes per point to a random place
+// shared-memory broadcasts (kFormDense).  The scatter writes 4 bytes per point to a random place
 // instead of 20 in five arrays (32-byte sectors: 5 of them; M = 3 10^7: 1.23
 // -> 0.21 ms); the coordinates are gathered here instead, and the records go
 // out in order (0.81 ms with the sort, M = 10^6 uniform without it: 21 us).  Bitonic sort of
@@ -531,7 +534,8 @@ constexpr int kRefinePer = kRefine / kRefineThreads;
 __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProblem* __restrict__ subs,
                                                            const int* __restrict__ num_subs, int* __restrict__ perm,
                                                            uint32_t* __restrict__ local, float* __restrict__ d0,
-                                                           float* __restrict__ d1, float* __restrict__ d2) {
+                                                           float* __restrict__ d1, float* __restrict__ d2,
+                                                           int* __restrict__ grid_points) {
   static_assert(kRefinePer == 4, "four elements per thread");
   __shared__ __align__(16) uint32_t key[kRefine];
   __shared__ uint32_t loc[kRefine];
@@ -548,7 +552,9 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
     n[t] = it.geom.n[t];
     bw[t] = it.geom.bin[t];
   }
-  int total_cells = 0;
+  int total_cells = 0, total_blocks = 0;   // of this thread's points, those that begin a cell, or planes of a slab
+  int first_plane = 0, last_plane = 0;
+  const int ahead = slab_ahead(it.win.taps);
   for (int r0 = 0; r0 < sub.count; r0 += kRefine) {
     const int cnt = min(kRefine, sub.count - r0), first = sub.start + r0;
     int size = 64;
@@ -587,7 +593,10 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
     }
     __syncthreads();
     // fewer points than cells: no run of the sort would be worth it
-    const int span = (int)((loc[cnt - 1] & 1023u) - (loc[0] & 1023u)) + 1;
+    const int l0 = (int)(loc[0] & 1023u);
+    last_plane = (int)(loc[cnt - 1] & 1023u);
+    if (r0 == 0) first_plane = l0;
+    const int span = last_plane - l0 + 1;
     if (cnt < span * bw[1] * bw[2]) {
 #pragma unroll
       for (int q = 0; q < kRefinePer; ++q) {
@@ -598,6 +607,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
         d1[first + i] = del[1][i];
         d2[first + i] = del[2][i];
         ++total_cells;
+        total_blocks += i == 0 || (int)(loc[i] & 1023u) / ahead != (int)(loc[i - 1] & 1023u) / ahead;
       }
       __syncthreads();
       continue;
@@ -646,6 +656,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
     int cells = 0;   // of this thread's points, those that begin a cell
     for (int i = threadIdx.x; i < cnt; i += kRefineThreads) {
       cells += i == 0 || key[i] >> 10 != key[i - 1] >> 10;
+      total_blocks += i == 0 || (int)(key[i] >> 20) / ahead != (int)(key[i - 1] >> 20) / ahead;
       const int p = (int)(key[i] & (kRefine - 1));
       perm[first + i] = idx[p];
       local[first + i] = loc[p];
@@ -657,12 +668,19 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(SortArgs s, SubProble
     __syncthreads();
   }
   // dense: kDenseRun points per occupied cell or more
-  __shared__ int occupied;
-  if (threadIdx.x == 0) occupied = 0;
+  __shared__ int occupied, blocks;
+  if (threadIdx.x == 0) occupied = blocks = 0;
   __syncthreads();
   atomicAdd(&occupied, total_cells);
+  atomicAdd(&blocks, total_blocks);
   __syncthreads();
-  if (threadIdx.x == 0) subs[blockIdx.x].dense = sub.count >= kDenseRun * occupied;
+  if (threadIdx.x == 0) {
+    const int planes = min(blocks * ahead, last_plane - first_plane + 1);   // of slabs
+    const bool slab = 2 * sub.count >= slab_points(it.win.taps) * planes;
+    const int form = sub.count >= kDenseRun * occupied ? kFormDense : (slab ? kFormSlab : kFormGrid);
+    subs[blockIdx.x].form = form;
+    if (form == kFormGrid) atomicAdd(&grid_points[sub.item], sub.count);
+  }
 }
 
 inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -732,22 +750,24 @@ int subproblem_launches(int nbins) { return nbins <= kSubSingle ? 1 : 2 + scan_l
 
 cudaError_t launch_subproblems(const SortArgs& s, const int* key_start, int P, int* bin_count, int* bin_start,
                                int* sub_count, int* sub_start, int* num_subs, int* partials, SubProblem* subs,
-                               cudaStream_t st) {
+                               int* grid_points, cudaStream_t st) {
   if (s.total_bins <= kSubSingle) {
-    k_subproblems<<<1, 1024, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_start, num_subs, subs);
+    k_subproblems<<<1, 1024, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_start, num_subs, subs,
+                                      grid_points);
     return cudaGetLastError();
   }
   k_sub_count<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, key_start, P, bin_count, bin_start, sub_count);
   const cudaError_t e = launch_scan(sub_count, sub_start, s.total_bins, num_subs, partials, false, st);
   if (e != cudaSuccess) return e;
-  k_sub_fill<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, bin_count, bin_start, sub_start, P, subs);
+  k_sub_fill<<<blocks_for(s.total_bins, 256), 256, 0, st>>>(s, bin_count, bin_start, sub_start, P, subs, grid_points);
   return cudaGetLastError();
 }
 
 cudaError_t launch_refine(const SortArgs& s, int64_t max_subs, SubProblem* subs, const int* num_subs, int* perm,
-                          uint32_t* local, float* const* delta, cudaStream_t st) {
+                          uint32_t* local, float* const* delta, int* grid_points, cudaStream_t st) {
   if (max_subs <= 0) return cudaSuccess;
-  k_refine<<<(unsigned)max_subs, kRefineThreads, 0, st>>>(s, subs, num_subs, perm, local, delta[0], delta[1], delta[2]);
+  k_refine<<<(unsigned)max_subs, kRefineThreads, 0, st>>>(s, subs, num_subs, perm, local, delta[0], delta[1], delta[2],
+                                                                  grid_points);
   return cudaGetLastError();
 }
 
