@@ -102,7 +102,9 @@ typedef enum {
   NFFT_OPT_MAX_SUBPROBLEM = 4,  /* points per subproblem (0 = default) */
   NFFT_OPT_RHS_CAPACITY = 5,    /* grids kept for right-hand sides processed together */
   NFFT_OPT_PROFILE = 6,         /* 1: record CUDA events around every stage */
-  NFFT_OPT_THREADS = 7,         /* threads per block of the point kernels (0 = default) */
+  NFFT_OPT_THREADS = 7,         /* threads per block of the point kernels (0 = default);
+                                   pencils (NFFT_METHOD_AUTO), grid-warp and tensor-core
+                                   kernels have fixed blocks and take no notice of it */
   NFFT_OPT_SPREAD_THREADS = 8,  /* threads per block of spreading only (overrides 7) */
   NFFT_OPT_INTERP_THREADS = 9,  /* threads per block of interpolation only (overrides 7) */
   NFFT_OPT_SPARSE_POINTS = 10,  /* with NFFT_METHOD_AUTO: spreading subproblems of

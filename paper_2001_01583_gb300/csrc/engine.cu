@@ -2041,7 +2041,10 @@ int Engine::autotune(int reps, double* best_ms) {
       continue;
     }
     double here = ranked[k].first;
-    for (int pass = 0; pass < 2; ++pass) {
+    // (pencils have blocks of their own: nothing to time)
+    bool threads = false;
+    for (const auto& kc : kclasses) threads = threads || !kc.pencil;
+    for (int pass = 0; threads && pass < 2; ++pass) {
       int& opt = pass == 0 ? spread_threads_opt : interp_threads_opt;
       int keep = 0;
       for (int th : {64, 128, 256}) {
