@@ -795,6 +795,7 @@ int Engine::build_layout() {
   const size_t K = (size_t)std::max(total_keys, 1);
   TRY(alloc_dev(key_count, sizeof(int) * K, device_bytes));
   CK(cudaMemset(key_count, 0, sizeof(int) * K));
+  keys_clear = true;
   TRY(alloc_dev(key_start, sizeof(int) * (K + 1), device_bytes));
   TRY(alloc_dev(bin_count, sizeof(int) * B, device_bytes));
   TRY(alloc_dev(bin_start, sizeof(int) * B, device_bytes));
@@ -1356,10 +1357,14 @@ int Engine::set_points_impl(const double* x_override) {
   s.single_d = items.size() == 1 ? items[0].geom.d : 0;
   EventPair ev{};
   TRY(stage_begin(NFFT_STAGE_SORT, &ev));
-  // (key_count is zero: the layout clears it, and so does every scan)
+  // key_count is zero: the layout clears it, and so does every scan; a call
+  // that failed between the two leaves counts behind
+  if (!keys_clear) CK(cudaMemsetAsync(key_count, 0, sizeof(int) * (size_t)std::max(total_keys, 1), stream));
+  keys_clear = false;
   CK(launch_key_count<Real>(s, key_count, key_rank, stream));
   kernel_launches += (s.total_points > 0 ? 2 : 0) + scan_launches(total_keys) + subproblem_launches(total_bins);
   CK(launch_scan(key_count, key_start, total_keys, key_start + total_keys, scan_partials, true, stream));
+  keys_clear = true;
   Real* d[3] = {static_cast<Real*>(delta[0]), static_cast<Real*>(delta[1]), static_cast<Real*>(delta[2])};
   CK(launch_scatter<Real>(s, key_start, key_rank, perm, local, d, stream));
   CK(launch_subproblems(s, key_start, max_sub, bin_count, bin_start, sub_count, sub_start, num_subs, scan_partials,

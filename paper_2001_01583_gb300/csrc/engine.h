@@ -206,6 +206,7 @@ class Engine {
   int64_t crop_blocks = 0, pad_blocks = 0;
   int* key_count = nullptr;       // points per sort key, and their exclusive scan
   int* key_start = nullptr;
+  bool keys_clear = false;        // key_count is zero, or will be after the work queued so far
   int* bin_count = nullptr;
   int* bin_start = nullptr;
   int* sub_count = nullptr;
