@@ -214,16 +214,19 @@ def _traffic(workload, stage):
 
 
 STAGE_KERNELS = {"spread": "k_spread_pencil (pencil layout) or k_spread_planes + k_spread_gm (bins), after a grid memset",
-                 "interp": "k_interp_pencil (pencil layout) or k_interp_groups + k_interp_gm (bins)",
+                 "interp": "k_interp_pencil (pencil layout; k_interp_gm for few points per plane) or "
+                           "k_interp_groups + k_interp_gm (bins)",
                  "sort": "k_key_count + k_scan + k_scatter + subproblem kernels + k_refine (pencil layout)",
                  "fft": "cuFFT C2C", "ifft": "cuFFT C2C", "deconv": "k_deconv_crop", "pad": "k_pad_deconv"}
 
 
-def _roofline(stages, workload, geom, peaks, kind, sms):
+def _roofline(stages, workload, geom, peaks, kind, sms, pencils=False):
     """The dominant stage's algorithmic HBM bytes per launch over its mean
     CUDA-event duration in the timed region, against the measured copy
-    bandwidth; the spreading and interpolation stages also against the
-    shared-memory pipe (a derived peak) and the FP32 pipe."""
+    bandwidth; the spreading and interpolation stages also against the FP32
+    pipe and, where their cells lie in shared memory (all but pencils: those
+    spread in registers and share reads), the shared-memory pipe (a derived
+    peak)."""
     N, M, sigma, taps, real = geom
     total = {k: v[0] for k, v in stages.items() if v[1] > 0}
     per_launch = {k: v[0] / v[1] for k, v in stages.items() if v[1] > 0}
@@ -250,12 +253,11 @@ def _roofline(stages, workload, geom, peaks, kind, sms):
         ach = visits * SMEM_BYTES_PER_CELL[st] / ts / 1e9
         # a complex value times a real weight added into a complex cell is two
         # FMAs (4 flops) per update, against 128 FP32 lanes x 2 flops per clock per SM
-        r["smem_pipe_" + st] = {"achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-                                "peak_kind": "derived: %d SMs x 128 B/clk x %.0f MHz" % (sms, mhz),
-                                "note": "bytes of a shared-memory tile's cell updates (pencil spreading updates "
-                                        "registers; pencil interpolation of dense bins shares its reads)",
-                                "cell_updates_per_s": visits / ts,
-                                "alu_fp32_frac": visits * 4 / ts / (sms * 128 * 2 * mhz * 1e6)}
+        r["cells_" + st] = {"cell_updates_per_s": visits / ts,
+                            "alu_fp32_frac": visits * 4 / ts / (sms * 128 * 2 * mhz * 1e6)}
+        if not pencils:
+            r["smem_pipe_" + st] = {"achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
+                                    "peak_kind": "derived: %d SMs x 128 B/clk x %.0f MHz" % (sms, mhz)}
     return r
 
 
@@ -633,7 +635,7 @@ def run_ours(args, wl, rank, world):
     props = torch.cuda.get_device_properties(dev)
     real = 4 if args.precision == "fp32" else 8
     roofline = _roofline(stages, args.workload, (N, M, sigma, taps, real), peaks, kind,
-                         props.multi_processor_count)
+                         props.multi_processor_count, pencils=len(N) == 3 and info["bin"][0] == 1023)
     hbm_step = len(xs) * _transform_bytes(N, M, sigma, 1, real)
     roofline["step_hbm_bytes"] = hbm_step
     roofline["step_hbm_frac"] = hbm_step / (ms_max * 1e-3) / 1e9 / peaks["hbm_gbs"]
