@@ -166,17 +166,18 @@ struct PencilLaunch {
 PencilLaunch pencil_launch_f32(int taps, bool spread);
 // Planes of points a slab serves.
 __host__ __device__ constexpr int slab_ahead(int taps) {
-  return taps == 6 || taps == 14 ? 12 : taps == 8 ? 9 : taps == 16 ? 14 : 7;
+  return taps == 14 ? 12 : taps == 6 || taps == 8 ? 9 : taps == 16 ? 14 : 7;
 }
 // Points per plane of a pencil (times two) from which interpolation loads slabs
 // of its planes; below, the grid-warp kernel reads the cells of each point
 // alone (W^3 of them; a slab is up to 24^2 cells per plane).  Where the two
 // meet.  Grid-warp / slabs, uniform points, N = 96^3, one right-hand side, us at
-// 1, 2, 4, 8 points per plane: 4 taps 26/42, 45/47, 69/53, 126/61; 6 taps 49/75,
-// 84/86, 150/102, 265/131; 8 taps 67/117, 121/131, 221/158, 434/214; 10 taps
+// 1, 2, 4, 8 points per plane: 4 taps 26/42, 45/47, 69/53, 126/61; 6 taps 49/79,
+// 84/96, 150/118, 265/137; 8 taps 67/117, 121/131, 221/158, 434/214; 10 taps
 // 226/238, 433/289, 838/391; 12 taps 88/167, 162/206, 281/275, 524/401; 14 taps
 // 170/272, 326/321, 644/414; 16 taps 243/374, 471/475, 860/658.  (N = 64^3 and
-// three right-hand sides meet a little higher for 4, 12 and 16 taps.)
+// three right-hand sides meet a little higher for 4, 12 and 16 taps, and lower
+// for 6: 39/35 us for N = 64^3 and 256/235 us for three, at 2 per plane.)
 __host__ __device__ constexpr int slab_points(int taps) {
   return taps <= 4 ? 6 : taps == 6 ? 4 : taps == 8 ? 5 : taps == 10 ? 2 : taps == 12 ? 10 : taps == 14 ? 4 : 6;
 }

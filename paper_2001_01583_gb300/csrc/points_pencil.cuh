@@ -383,8 +383,9 @@ struct SlabShape {
   // points: more planes mean fewer reloads and fewer resident blocks.  8 taps,
   // uniform, M = 10^6: 254 us for 3 planes, 236 for 4, 213 for 7, 206 for 9, 210
   // for 12; 96000 points, three right-hand sides: 346, 259, 219, 195, 180.
-  // N = 96^3, one right-hand side, 2 / 8 points per plane: 6 taps 105 / 151 us
-  // for 7 planes, 86 / 131 for 12; 12 taps 459 / 634 for 2 planes and 256 threads,
+  // N = 96^3, one right-hand side, 2 / 8 points per plane: 6 taps 102 / 151 us
+  // for 7 planes, 96 / 137 for 9, 83 / 133 for 12, which takes dense subproblems
+  // longer (the largest configuration 2.02 ms for 7, 2.09 for 12); 12 taps 459 / 634 for 2 planes and 256 threads,
   // 206 / 401 for 7 and 128, 217 / 428 for 12 and 256; 14 taps 1077 / 1627 for 1
   // and 128, 538 / 854 for 4 and 256, 321 / 623 for 12 and 256; 16 taps 1791 / 2628
   // for 1 and 128, 588 / 1126 for 8 and 256, 475 / 1006 for 14 and 256; 10 taps
